@@ -368,11 +368,10 @@ int compile(musr_ctx* ctx, int prec, int var) {
       hs.dkt_span = std::max(hs.dkt_span, (static_cast<double>(ctx->nhi[h] - 1) - ctx->t0[h]) * ctx->dt_us);
   std::vector<std::vector<int>> groups;
   int group_cap = 1;
-  const bool basis = prec == MUSR_SPLIT &&
-                     !musr::plan_split(ctx->terms.data(), hs.nterms, ctx->map.data(), H, ctx->nslots,
+  const bool basis = !musr::plan_split(ctx->terms.data(), hs.nterms, ctx->map.data(), H, ctx->nslots,
                                        ctx->consts.data(), &hs, !ctx->asym);
-  if (prec == MUSR_SPLIT && !basis) {  // the term list per bin in FP32
-    bool small = hs.nterms <= 2;
+  if (!basis) {  // the term list per bin (FP32 on the SPLIT path, with a smaller kernel for short lists)
+    bool small = prec == MUSR_SPLIT && hs.nterms <= 2;
     for (int k = 0; k < hs.nterms; ++k) small = small && ctx->terms[k].nprim <= 3;
     hs.shape = small ? musr::kShapeListS : musr::kShapeList;
   }
@@ -397,10 +396,11 @@ int compile(musr_ctx* ctx, int prec, int var) {
     for (int h = 0; h < H; ++h) {
       std::vector<int64_t> key;
       int64_t tb;
-      // t0 to 2^-24 bins: a smaller difference in time zero (below 2^-24 bin widths in
-      // every time) is far below the FP32 resolution of the shared per-bin factors
+      // t0 to 2^-24 bins on the SPLIT path: a smaller difference in time zero (below 2^-24 bin
+      // widths in every time) is far below the FP32 resolution of the shared per-bin factors;
+      // the FP64 path shares them between equal t0 only
       const double q = std::nearbyint(ctx->t0[h] * 16777216.0);
-      if (std::fabs(q) < 4e18) {
+      if (prec == MUSR_SPLIT && std::fabs(q) < 4e18) {
         key.push_back(0);
         key.push_back(static_cast<int64_t>(q));
       } else {
@@ -463,7 +463,7 @@ int compile(musr_ctx* ctx, int prec, int var) {
     col += ch.nh * ctx->nslots;
   }
   hs.group = group_cap;
-  hs.nch = prec == MUSR_SPLIT ? musr::shape_channels(hs.shape) : musr::kFp64Channels;
+  hs.nch = musr::shape_channels(hs.shape);
   hs.pstride = 1 + hs.nch;
   hs.ncols = col;
   hs.nchunks = static_cast<int>(chunks.size());
@@ -579,6 +579,10 @@ int pick_variant(musr_ctx* ctx, int prec, int nvec) {
     ensure_compiled(ctx, prec, v);
     items[v] = ctx->comp[prec][v].hs.nitems;
   }
+  const HistSet& hs = ctx->comp[prec][0].hs;
+  if (prec == MUSR_FP64 && hs.shape != musr::kShapeList)
+    return musr::pick_decomposition(items, nvec, musr::persistent_grid(prec, ctx->num_sms),
+                                    musr::fp64_basis_item_cost(ctx->comp[prec][0].chunks[0].nh));
   return musr::pick_decomposition(items, nvec, prec, ctx->num_sms);
 }
 

@@ -10,10 +10,10 @@
 //     job's last item sums that job's rows in a fixed order (deterministic: the
 //     result does not depend on which CTA ran which item, nor on other jobs).
 //
-// FP64 path: a chunk is one histogram.  SPLIT path: a chunk is up to
-// kGroupMax histograms that share t0 and every time-dependent parameter
-// (relaxation rates, Kubo-Toyabe width, frequencies), so that the time-only
-// factors of a bin are evaluated once and reused across the chunk.
+// A chunk is up to kGroupMax histograms that share t0 and every time-dependent parameter
+// (relaxation rates, Kubo-Toyabe width, frequencies), so that the time-only factors of a bin
+// are evaluated once and reused across the chunk; one histogram where the theory has no basis
+// form.
 #pragma once
 
 #include <cstdint>
@@ -85,18 +85,18 @@ enum Shape : int {
   kShapeT2N1 = 5,     // two cosine terms + other (M = 6)
   kShapeT2m = 6,      // merged two cosine terms (M = 3)
   kShapeT2N1m = 7,    // merged two cosine terms + other (M = 3)
-  kShapeList = 8,     // no basis form: the term list per bin in FP32 (one histogram per chunk)
+  kShapeList = 8,     // no basis form: the term list per bin (one histogram per chunk)
   kShapeListS = 9     // the same for at most 2 terms of at most 3 primitives (fewer registers)
 };
 
-// A term as given: the product of nprim primitives (FP64 path).
+// A term as given: the product of nprim primitives (the term-list kernels).
 struct RawTerm {
   int nprim;
   int kind[kMaxPrims];
   int slot[kMaxPrims][2];
 };
 
-// A term in canonical form (SPLIT path):
+// A term in canonical form (the basis kernels):
 //   a * exp(-Lambda t - S t^2 / 2) * [KT(Delta, t) or LKT(a, t)] * [cos(2 pi (nu t + phi / 360))]
 // with Lambda the sum of its EXP rates and S the sum of its squared GAUSS widths.
 struct CanonTerm {
@@ -301,6 +301,10 @@ inline int pick_decomposition(const int* items, int64_t nvec, int grid, double i
 // SPLIT kernels run two CTAs per SM, the FP64 kernels one.
 constexpr double kSplitItemCost = 1.3;
 constexpr double kFp64ItemCost = 0.1;
+// The FP64 basis kernels: an item costs about 200 FP64 instructions per thread (fresh time
+// factors, the channels' warp sums), an iteration 25 per histogram of the chunk and 20 for the
+// time factors.
+inline double fp64_basis_item_cost(int nh) { return 200.0 / (25.0 * (nh > 0 ? nh : 1) + 20.0); }
 inline int persistent_grid(int precision, int num_sms) { return num_sms * (precision == 1 ? 2 : 1); }
 inline int pick_decomposition(const int* items, int64_t nvec, int precision, int num_sms) {
   return pick_decomposition(items, nvec, persistent_grid(precision, num_sms),

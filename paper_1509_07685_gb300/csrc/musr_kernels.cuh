@@ -9,9 +9,10 @@
 // No tensor cores: nothing here is a contraction.
 //
 // Two paths:
-//   * FP64 ("plain"): one work item is a tile of one histogram; every per-bin
-//     operation in FP64, the term list interpreted as given (any product of
-//     primitives).
+//   * FP64 ("plain"): theories with a basis form run musr_kernels_f64.cuh (chunks of up to 8
+//     histograms, every operation in FP64).  For the others (and in the allocation-free entry
+//     point) one work item is a tile of one histogram, every per-bin operation in FP64, the
+//     term list interpreted as given (any product of primitives).
 //   * SPLIT: one work item is a tile of a chunk of <= 8 histograms that share
 //     the time grid and every time-dependent parameter.  For each bin the
 //     time-only factors (muon decay, relaxations, Kubo-Toyabe, the precession's
@@ -1700,8 +1701,8 @@ __device__ void finish_chunk(const Job& job, const HistSet& hs, SM& sm) {
 // CTA barrier orders every thread's row writes before thread 0's acquire-release counter
 // increment (cumulative over what the barrier ordered before it); acquire: that same
 // atomic, and a fence by every thread of the finalizing CTA.
-template <int PREC, int SHAPE, bool GRAD>
-__device__ void complete_item(const Job& job, const HistSet& hs, Smem& sm) {
+template <int PREC, int SHAPE, bool GRAD, class SM>
+__device__ void complete_item(const Job& job, const HistSet& hs, SM& sm) {
   __syncthreads();
   if (threadIdx.x == 0) {
     const unsigned prev = atom_add_acq_rel(job.chunk_count + sm.cc.chunk, 1u);
@@ -1877,5 +1878,12 @@ MUSR_DECLARE_GROUP(a)
 MUSR_DECLARE_GROUP(b)
 MUSR_DECLARE_GROUP(c)
 #undef MUSR_DECLARE_GROUP
+// The FP64 basis kernels (musr_kernels_f64.cuh), by the same groups of shapes.
+int launch_group_f64_a(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
+                       LaunchInfo* info);
+int launch_group_f64_b(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
+                       LaunchInfo* info);
+int launch_group_f64_c(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
+                       LaunchInfo* info);
 
 }  // namespace musr

@@ -160,6 +160,7 @@ extern "C" int musr_eval_noalloc(const void* d_counts, int dtype, int nhist, int
   // Theories without a basis form evaluate their term list per bin in FP32 (one histogram
   // per chunk), as a context does.
   const bool basis = precision == MUSR_SPLIT && !plan_split(terms, nterms, map, nhist, nslots, consts, &hs);
+  if (precision == MUSR_FP64) hs.shape = kShapeList;  // the term list, one histogram per chunk
   if (precision == MUSR_SPLIT && !basis) {
     bool small = nterms <= 2;
     for (int k = 0; k < nterms; ++k) small = small && terms[k].nprim <= 3;
