@@ -299,6 +299,8 @@ void free_compiled(musr_ctx* ctx, Compiled& c) {
   c.uploaded = false;
   c.chunks.clear();
   c.items.clear();
+  c.slot_src.clear();
+  c.chunk_hist.clear();
   c.hist_index.clear();
   c.col_chunk.clear();
   c.p_ptr.clear();
@@ -470,6 +472,14 @@ int compile(musr_ctx* ctx, int prec, int var) {
   hs.nitems = static_cast<int>(items.size());
   std::vector<int> col_chunk(std::max(col, 1));
   std::vector<std::vector<int>> pcols(ctx->P);
+  // Columns of the basis kernels that are always 0: a slot with time-only derivatives alone (they
+  // are the chunk's, in its first histogram's columns) or with none, in the other histograms.
+  auto always_zero = [&](int hl, int s) {
+    if (!basis || hl == 0) return false;
+    for (int e = hs.slot_ptr[s]; e < hs.slot_ptr[s + 1]; ++e)
+      if (hs.contrib[hs.slot_list[e]].kind < musr::kCLam) return false;
+    return true;
+  };
   for (size_t ci = 0; ci < chunks.size(); ++ci) {
     const Chunk& ch = chunks[ci];
     for (int hl = 0; hl < ch.nh; ++hl) {
@@ -478,7 +488,7 @@ int compile(musr_ctx* ctx, int prec, int var) {
         const int cc = ch.col0 + hl * ctx->nslots + s;
         col_chunk[cc] = static_cast<int>(ci);
         const int32_t m = ctx->map[static_cast<size_t>(h) * ctx->nslots + s];
-        if (m >= 0) pcols[m].push_back(cc);
+        if (m >= 0 && !always_zero(hl, s)) pcols[m].push_back(cc);
       }
     }
   }
@@ -495,6 +505,16 @@ int compile(musr_ctx* ctx, int prec, int var) {
   c.dkt_of = std::move(dkt_of);
   c.chunks = std::move(chunks);
   c.items = std::move(items);
+  c.slot_src.assign(c.chunks.size() * musr::kGroupMax * std::max(ctx->nslots, 1), 0);
+  c.chunk_hist.assign(c.chunks.size() * musr::kGroupMax, -1);
+  for (size_t ci = 0; ci < c.chunks.size(); ++ci)
+    for (int hl = 0; hl < c.chunks[ci].nh; ++hl) {
+      const int h = hist_index[c.chunks[ci].first + hl];
+      const size_t at = ci * musr::kGroupMax + hl;
+      c.chunk_hist[at] = h;
+      for (int s = 0; s < ctx->nslots; ++s)
+        c.slot_src[at * ctx->nslots + s] = ctx->map[static_cast<size_t>(h) * ctx->nslots + s];
+    }
   c.hist_index = std::move(hist_index);
   c.col_chunk = std::move(col_chunk);
   c.p_ptr = std::move(p_ptr);
@@ -536,6 +556,8 @@ int ensure_uploaded(musr_ctx* ctx, int prec, int var) {
   const size_t o_mp = place(sizeof(int32_t) * ctx->map.size());
   const size_t o_cs = place(sizeof(double) * nconsts);
   const size_t o_dk = place(sizeof(int) * std::max<size_t>(c.dkt_of.size(), 1));
+  const size_t o_ss = place(sizeof(int32_t) * c.slot_src.size());
+  const size_t o_sh = place(sizeof(int) * c.chunk_hist.size());
   int rc = dalloc(ctx, c.tables, off);
   if (rc) return rc;
   char* base = static_cast<char*>(c.tables.p);
@@ -549,6 +571,8 @@ int ensure_uploaded(musr_ctx* ctx, int prec, int var) {
   hs.map = reinterpret_cast<const int32_t*>(base + o_mp);
   hs.consts = reinterpret_cast<const double*>(base + o_cs);
   hs.dkt_of = reinterpret_cast<const int*>(base + o_dk);
+  hs.slot_src = reinterpret_cast<const int32_t*>(base + o_ss);
+  hs.chunk_hist = reinterpret_cast<const int*>(base + o_sh);
   std::vector<char>& blob = c.blob;  // kept until the tables are freed: the copy's source
   blob.assign(off, 0);
   std::memcpy(blob.data() + o_hs, &hs, sizeof(hs));
@@ -560,6 +584,8 @@ int ensure_uploaded(musr_ctx* ctx, int prec, int var) {
   std::memcpy(blob.data() + o_pc, c.p_cols.data(), sizeof(int) * c.p_cols.size());
   std::memcpy(blob.data() + o_mp, ctx->map.data(), sizeof(int32_t) * ctx->map.size());
   if (!ctx->consts.empty()) std::memcpy(blob.data() + o_cs, ctx->consts.data(), sizeof(double) * ctx->consts.size());
+  std::memcpy(blob.data() + o_ss, c.slot_src.data(), sizeof(int32_t) * c.slot_src.size());
+  std::memcpy(blob.data() + o_sh, c.chunk_hist.data(), sizeof(int) * c.chunk_hist.size());
   if (!c.dkt_of.empty()) std::memcpy(blob.data() + o_dk, c.dkt_of.data(), sizeof(int) * c.dkt_of.size());
   cudaError_t e = cudaMemcpyAsync(base, blob.data(), off, cudaMemcpyHostToDevice,
                                   ctx->setup_stream ? ctx->setup_stream : ctx->stream);
@@ -636,6 +662,7 @@ void fill_jobs(musr_ctx* ctx, int prec, int var, int mode, int grad, int nvec, c
     j.hs = d_hs;
     j.params = d_params + static_cast<size_t>(v) * ctx->P;
     j.out = d_out + static_cast<size_t>(v) * (1 + ctx->P);
+    j.items = hs.items;
     j.partials = static_cast<double*>(ev.partials.p) + static_cast<size_t>(v) * hs.nitems * hs.pstride;
     j.nrows = hs.nitems;
     j.colsum = static_cast<double*>(ev.colsum.p) + static_cast<size_t>(v) * std::max(hs.ncols, 1);
@@ -755,6 +782,7 @@ int prepare_jobs(musr_ctx* ctx, int prec, int var, int mode, int grad, int nvec,
   }
   e = copy_h2d(ev.jobs.p, jobs.data(), sizeof(Job) * nvec);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpyAsync(jobs)");
+  ev.first = jobs[0];
   ev.key_valid = true;
   ev.k_prec = prec;
   ev.k_var = var;
@@ -790,6 +818,7 @@ struct LaunchPlan {
   bool empty = false, pieces = false;
   int grid = 0;
   double* d_out = nullptr;
+  const double* x = nullptr;  // one evaluation's parameters (host), to go with the launch
 };
 
 int plan_launch(musr_ctx* ctx, int prec, int mode, int grad, int nvec, const double* d_params, double* d_out,
@@ -834,8 +863,13 @@ int issue_launch(musr_ctx* ctx, const LaunchPlan& L) {
     ctx->ev.key_valid = false;
     return cuda_fail(ctx, e, "dynamic Kubo-Toyabe table launch");
   }
-  if (musr::launch_eval(L.prec, hs.shape, L.mode, L.grad, static_cast<const Job*>(ctx->ev.jobs.p), L.nvec,
-                        L.pieces ? L.grid : L.nvec * hs.nitems, ctx->num_sms, ctx->stream, &info)) {
+  musr::LaunchHead head{static_cast<const Job*>(ctx->ev.jobs.p), L.nvec, L.pieces ? L.grid : L.nvec * hs.nitems,
+                        hs.nitems, 0, ctx->ev.first, {}};
+  if (L.x) {
+    head.nx = ctx->P;
+    std::memcpy(head.x, L.x, sizeof(double) * ctx->P);
+  }
+  if (musr::launch_eval(L.prec, hs.shape, L.mode, L.grad, head, ctx->num_sms, ctx->stream, &info)) {
     cudaError_t e = cudaGetLastError();
     ctx->ev.key_valid = false;
     return cuda_fail(ctx, e, "kernel launch");
@@ -1308,21 +1342,28 @@ int musr_eval_batch(musr_ctx* ctx, const double* params, int nvec, int nparams, 
     if ((rc = dalloc(ctx, ev.params, std::max<size_t>(np, 1) * sizeof(double)))) return rc;
     ev.key_valid = false;
   }
-  if (ev.out.bytes < no * sizeof(double)) {
-    if ((rc = dalloc(ctx, ev.out, no * sizeof(double)))) return rc;
-    ev.key_valid = false;
-  }
   const int grad = out_grads != nullptr;
-  std::memcpy(ev.h_in, params, np * sizeof(double));
   LaunchPlan L;
-  if ((rc = plan_launch(ctx, precision, mode, grad, nvec, static_cast<const double*>(ev.params.p),
-                        static_cast<double*>(ev.out.p), nullptr, &L)))
+  // The kernels write values and gradients straight into the pinned buffer the host reads (each job's
+  // 1 + P values once, at its end), and a single evaluation's parameters go with its launch: no copy
+  // before or after the kernel (GB300: about 3 us of a 33 us call).
+  if ((rc = plan_launch(ctx, precision, mode, grad, nvec, static_cast<const double*>(ev.params.p), ev.h_out, nullptr,
+                        &L)))
     return rc;
-  cudaError_t e = cudaMemcpyAsync(ev.params.p, ev.h_in, np * sizeof(double), cudaMemcpyHostToDevice, ctx->stream);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpyAsync(params)");
-  if ((rc = issue_launch(ctx, L))) return rc;
-  e = cudaMemcpyAsync(ev.h_out, ev.out.p, no * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpyAsync(out)");
+  cudaError_t e = cudaSuccess;
+  if (L.empty) {
+    std::memset(ev.h_out, 0, no * sizeof(double));
+  } else {
+    // the table solve of a dynamic Kubo-Toyabe factor reads the parameters from the device
+    if (nvec == 1 && P <= musr::kHeadParams && ctx->comp[precision][L.var].hs.ndkt == 0) {
+      L.x = params;
+    } else {
+      std::memcpy(ev.h_in, params, np * sizeof(double));
+      e = cudaMemcpyAsync(ev.params.p, ev.h_in, np * sizeof(double), cudaMemcpyHostToDevice, ctx->stream);
+      if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpyAsync(params)");
+    }
+    if ((rc = issue_launch(ctx, L))) return rc;
+  }
   e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaStreamSynchronize");
   bool nonfinite = false;

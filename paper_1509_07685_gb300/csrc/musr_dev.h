@@ -146,7 +146,7 @@ struct Chunk {
   double t0;      // time-zero bin shared by the chunk
 };
 
-struct HistSet {
+struct alignas(16) HistSet {  // copied by 16-byte words into shared memory
   // histograms: [H][stride] in FP32 or FP64
   const void* counts;
   int store;
@@ -167,6 +167,8 @@ struct HistSet {
   float bamp[kMaxTerms];       // SPLIT basis amplitude of each term (its constant if merged, else 1)
   int ncontrib;
   Contrib contrib[kMaxContrib];
+  // the contributions of slot s, in order: contrib[slot_list[slot_ptr[s] .. slot_ptr[s + 1])]
+  unsigned char slot_ptr[kMaxSlots + 1], slot_list[kMaxContrib];
   // dynamic Kubo-Toyabe sources: map entries of (Delta, nu) of each, and per (histogram,
   // term, primitive) the source index or -1 ([H][kMaxTerms][kMaxPrims]); span of the tables
   int ndkt;
@@ -184,6 +186,11 @@ struct HistSet {
   int nchunks;
   const int* hist_index;   // histograms of the chunks, chunk by chunk
   const int2* items;       // (chunk, tile) per work item
+  // per chunk, so that a CTA needs no table to find the next: the map entries of its histograms
+  // ([nchunks][kGroupMax][nslots], 0 beyond the chunk's) and the histograms ([nchunks][kGroupMax],
+  // -1 beyond); nullptr: through hist_index and map
+  const int32_t* slot_src;
+  const int* chunk_hist;
   int nitems;
   int tile_bins;           // bins per tile
   int group;               // histograms per chunk at most
@@ -206,6 +213,7 @@ struct Job {
   const HistSet* hs;
   const double* params;      // [P]
   double* out;               // [1 + P]
+  const int2* items;         // hs->items
   double* partials;          // [nrows][hs->pstride]
   int nrows;                 // partial rows of this job: hs->nitems, or its pieces' count
   double* colsum;            // [hs->ncols]
@@ -244,13 +252,26 @@ enum DebugCheck : unsigned {
   kDbgJob = 128u      // a job index beyond the launch's jobs
 };
 
+// What a launch's kernel gets by value: the jobs on the device, their number, the launch's
+// work items (its CTAs with a launch-level partition), the items of every job where the jobs share
+// one histogram set (0: they do not), and the first job itself (a single evaluation reads no job
+// from memory).
+// x: the parameters of a launch of one job that come with it (nx of them; 0: at first.params).
+constexpr int kHeadParams = 128;
+struct LaunchHead {
+  const Job* jobs;
+  int njobs, total_items, per_job, nx;
+  Job first;
+  double x[kHeadParams];
+};
+
 // Launchers (host side of musr_kernels.cu).  All enqueue on `stream`.
 struct LaunchInfo {
   int grid;
   int block;
 };
-int launch_eval(int precision, int shape, int mode, int grad, const Job* d_jobs, int njobs,
-                int total_items, int num_sms, void* stream, LaunchInfo* info);
+int launch_eval(int precision, int shape, int mode, int grad, const LaunchHead& head, int num_sms, void* stream,
+                LaunchInfo* info);
 int max_ctas_per_sm(int precision, int shape, int mode, int grad);
 // The dynamic Kubo-Toyabe tables of njobs evaluations of one histogram set (precision 0:
 // FP64, 1: FP32), two CTAs per (job, source); enqueued on `stream` before the evaluation.

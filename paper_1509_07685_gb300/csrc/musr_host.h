@@ -58,6 +58,8 @@ struct Compiled {
   std::vector<Chunk> chunks;
   std::vector<int2> items;
   std::vector<int> hist_index, col_chunk, p_ptr, p_cols;
+  std::vector<int32_t> slot_src;  // [nchunks][kGroupMax][nslots] map entries by chunk
+  std::vector<int> chunk_hist;    // [nchunks][kGroupMax] histograms by chunk, -1 beyond
   std::vector<int> dkt_of;  // [H][kMaxTerms][kMaxPrims] dynamic Kubo-Toyabe source or -1
   bool uploaded = false;
   DevBuf tables;        // HistSet + all tables + map + consts, 256-byte aligned pieces
@@ -74,6 +76,7 @@ struct EvalBufs {
   double* h_in = nullptr;
   double* h_out = nullptr;
   size_t h_in_bytes = 0, h_out_bytes = 0;
+  Job first{};           // the first job of the table on the device (launches carry it)
   bool key_valid = false;
   int k_prec = -1, k_var = -1, k_mode = -1, k_grad = -1, k_nvec = -1;
   const double* k_params = nullptr;

@@ -58,27 +58,27 @@ int shape_channels(int shape) {
   }
 }
 
-int launch_eval(int precision, int shape, int mode, int grad, const Job* d_jobs, int njobs,
-                int total_items, int num_sms, void* stream, LaunchInfo* info) {
+int launch_eval(int precision, int shape, int mode, int grad, const LaunchHead& head, int num_sms, void* stream,
+                LaunchInfo* info) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (precision == 0) {  // the basis kernels where the theory has a basis form, else the term list
-    if (shape == kShapeList) return launch_group_fp64(mode, grad, d_jobs, njobs, total_items, num_sms, s, info);
+    if (shape == kShapeList) return launch_group_fp64(mode, grad, head, num_sms, s, info);
     switch (shape_group_of(shape)) {
       case 1:
-        return launch_group_f64_b(shape, mode, grad, d_jobs, njobs, total_items, num_sms, s, info);
+        return launch_group_f64_b(shape, mode, grad, head, num_sms, s, info);
       case 2:
-        return launch_group_f64_c(shape, mode, grad, d_jobs, njobs, total_items, num_sms, s, info);
+        return launch_group_f64_c(shape, mode, grad, head, num_sms, s, info);
       default:
-        return launch_group_f64_a(shape, mode, grad, d_jobs, njobs, total_items, num_sms, s, info);
+        return launch_group_f64_a(shape, mode, grad, head, num_sms, s, info);
     }
   }
   switch (shape_group_of(shape)) {
     case 1:
-      return launch_group_b(shape, mode, grad, d_jobs, njobs, total_items, num_sms, s, info);
+      return launch_group_b(shape, mode, grad, head, num_sms, s, info);
     case 2:
-      return launch_group_c(shape, mode, grad, d_jobs, njobs, total_items, num_sms, s, info);
+      return launch_group_c(shape, mode, grad, head, num_sms, s, info);
     default:
-      return launch_group_a(shape, mode, grad, d_jobs, njobs, total_items, num_sms, s, info);
+      return launch_group_a(shape, mode, grad, head, num_sms, s, info);
   }
 }
 

@@ -141,18 +141,41 @@ __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned v) {
   asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
   return old;
 }
-__device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
-__device__ __forceinline__ float warp_sum_f(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// Sums a[0 .. N) over the warp's lanes, N a multiple of 32: a lane keeps N / 32 of the sums (lane
+// l the entries l N / 32 ..., in a[0 .. N / 32)).  Each step adds half of what is left, N - N / 32
+// additions per warp where a butterfly per entry takes 5 N; every entry is summed in the order
+// (and to the bits) of a butterfly (warp_sum_d).
+template <int N, class T>
+__device__ __forceinline__ void warp_scatter_sum(T (&a)[N]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16, n = N / 2; o > 0; o >>= 1, n >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+      if (i >= n) break;
+      const T keep = up ? a[i + n] : a[i], send = up ? a[i] : a[i + n];
+      a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+}
+// A float as a double on the integer pipe (a conversion instruction would occupy the FP64
+// pipe); subnormal floats, which counts never are, take the conversion.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f);
+  const unsigned e = b & 0x7f800000u;
+  if (e == 0u && (b & 0x007fffffu)) return static_cast<double>(f);
+  const unsigned bias = e == 0x7f800000u ? 0x70000000u : 0x38000000u;  // infinity and NaN keep their exponent
+  const unsigned hi = (b & 0x80000000u) | (e ? ((b & 0x7fffffffu) >> 3) + bias : 0u);
+  return __hiloint2double(static_cast<int>(hi), static_cast<int>(b << 29));
+}
+
 // Warp sum of a float-float pair (hi, lo): Knuth's TwoSum on the hi parts.
 __device__ __forceinline__ void warp_sum_ff(float& hi, float& lo) {
 #pragma unroll
@@ -272,21 +295,32 @@ struct TileState {
   float lbase[kMaxTerms * kMaxPrims];
 };
 
+// A job's finalisation (job_finalize): the warps' sums of chunk values, and for a job of one chunk
+// its columns and the parameters' lists of columns, fetched while its rows are summed.
+struct Finish {
+  double wsum[kWarps];
+  double cols[kGroupMax * kMaxSlots];
+  int p_ptr[kBlock], p_cols[kBlock];
+};
+
 struct Smem {
   // SPLIT, FP32 counts: the rows of the current and the next CTA iteration, each thread's two
   // bins of every histogram copied by that thread (cp.async)
   alignas(128) float stage[2][kGroupMax][kBlock * kBinsPerThread];
   __device__ float* stage_slot(int b, int hl, int bin) { return &stage[b][hl][bin]; }
+  Job job;                       // the current job and its histogram set (enter_job)
+  double x[kHeadParams];         // its parameters, where the launch brings them
+  HistSet hs;
+  const HistSet* hs_src;         // where hs was copied from
   ChunkCache cc;
   TileState ts;
+  Finish fin;
   float dkn[kMaxTerms][kBinsPerThread][kBlock];  // d/dnu factors of dynamic Kubo-Toyabe terms, per thread
   float cred[kWarps][kMaxChan];  // per-warp FP32 channel sums
   float vred[kWarps][2];         // per-warp float-float value
-  double dred[kWarps][kFp64Channels + 2];
+  double dred[kWarps][kFp64Channels + 2];  // also the half sums of split_item (64 of them)
   double tot[kMaxChan + 1];      // chunk totals in the chunk finalize
-  double wsum[kWarps];
   int flag;
-  int bad;
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -352,43 +386,77 @@ __device__ __forceinline__ void phase_cs(double phi_deg, double* c, double* s) {
   *s = sf;
 }
 
-// Coefficients [Nbkg, Gam_0 .. Gam_{M-1}] of one histogram's basis expansion from its slot
-// values slot(s), computed in FP64 and rounded once; cos and sin of each cosine term's phase.
+// Term k's part of the coefficients [Nbkg, Gam_0 .. Gam_{M-1}] of one histogram's basis expansion
+// (term 0 with Nbkg and N0), from its slot values slot(s), computed in FP64 and rounded once; cos
+// and sin of a cosine term's phase.  A lane per (histogram, term): an FP64 warp instruction holds
+// its sub-partition's pipe for 64 clocks whatever the lanes in it, so a set-up is as long as its
+// chain of FP64 instructions.
 template <int SHAPE, class Slot>
-__device__ void coef_row(const HistSet& hs, Slot slot, float* gam, double* cph, double* sph) {
+__device__ __forceinline__ void coef_term(const HistSet& hs, Slot slot, int k, float* gam, double* cph, double* sph) {
   using Bs = Basis<SHAPE>;
-  double g[kGamStride];
-#pragma unroll
-  for (int i = 0; i < kGamStride; ++i) g[i] = 0.0;
   const double N0 = slot(0);
-  g[0] = slot(1);
-  g[1] = hs.envelope ? N0 : 0.0;  // the basis function E carries the 1 of (1 + A)
-#pragma unroll
-  for (int k = 0; k < kMaxTerms; ++k) {
-    double c = 1.0, sn = 0.0;
-    if (k < hs.nterms && hs.canon[k].kind == kTermTF) phase_cs(slot(hs.canon[k].phi_slot), &c, &sn);
-    cph[k] = c;
-    sph[k] = sn;
+  double c = 1.0, sn = 0.0;
+  const bool live = k < hs.nterms;
+  const int kind = live ? hs.canon[k].kind : kTermNone;
+  if (kind == kTermTF) phase_cs(slot(hs.canon[k].phi_slot), &c, &sn);
+  cph[k] = c;
+  sph[k] = sn;
+  if (k == 0) {
+    gam[0] = static_cast<float>(slot(1));
+    gam[1] = hs.envelope ? static_cast<float>(N0) : 0.0f;  // the basis function E carries the 1 of (1 + A)
   }
   if (Bs::MERGED) {  // one phase per histogram: that of the first cosine term
-    g[2] = N0 * cph[0];
-    g[3] = -N0 * sph[0];
-  } else {
+    if (k == 0) {
+      gam[2] = static_cast<float>(N0 * c);
+      gam[3] = static_cast<float>(-N0 * sn);
+    }
+  } else if (k < Bs::NT) {
+    const int amp = live ? hs.canon[k].amp_slot : -1;
+    const double a = amp >= 0 ? slot(amp) : 1.0;
+    const double Na = live ? N0 * a : 0.0;
+    gam[1 + Bs::bc(k)] = static_cast<float>(kind == kTermTF ? Na * c : Na);
+    if (Bs::NTF < 0 || k < Bs::NTF) gam[1 + Bs::bs(k)] = kind == kTermTF ? static_cast<float>(-Na * sn) : 0.0f;
+  }
+}
+
+// Directional derivative of histogram hl's coefficients along a Gauss-Newton direction.
+template <int SHAPE>
+__device__ void gdot_row(const Job& job, const HistSet& hs, int hl, ChunkCache& cc) {
+  using Bs = Basis<SHAPE>;
+  double gd[kGamStride];
 #pragma unroll
-    for (int k = 0; k < Bs::NT; ++k) {
-      if (k >= hs.nterms) break;
-      const CanonTerm& ct = hs.canon[k];
-      const double a = ct.amp_slot >= 0 ? slot(ct.amp_slot) : 1.0;
-      if (ct.kind == kTermTF) {
-        g[1 + Bs::bc(k)] = N0 * a * cph[k];
-        g[1 + Bs::bs(k)] = -N0 * a * sph[k];
-      } else {
-        g[1 + Bs::bc(k)] = N0 * a;
+  for (int i = 0; i < kGamStride; ++i) gd[i] = 0.0;
+  if (job.dir) {
+    constexpr double kDeg = kTwoPi / 360.0;
+    const double N0 = cc.loc[hl][0], vN0 = cc.ldir[hl][0];
+    gd[0] = cc.ldir[hl][1];
+    gd[1] = hs.envelope ? vN0 : 0.0;
+    if (Bs::MERGED) {
+      const double vph = cc.ldir[hl][hs.canon[0].phi_slot] * kDeg;
+      const double c = cc.cph[hl][0], sn = cc.sph[hl][0];
+      gd[2] = vN0 * c - N0 * sn * vph;
+      gd[3] = -vN0 * sn - N0 * c * vph;
+    } else {
+#pragma unroll
+      for (int k = 0; k < Bs::NT; ++k) {
+        if (k >= hs.nterms) break;
+        const CanonTerm& ct = hs.canon[k];
+        const double a = ct.amp_slot >= 0 ? cc.loc[hl][ct.amp_slot] : 1.0;
+        const double va = ct.amp_slot >= 0 ? cc.ldir[hl][ct.amp_slot] : 0.0;
+        const double dNa = vN0 * a + N0 * va;  // d(N0 a) along v
+        if (ct.kind == kTermTF) {
+          const double vph = cc.ldir[hl][ct.phi_slot] * kDeg;
+          const double c = cc.cph[hl][k], sn = cc.sph[hl][k];
+          gd[1 + Bs::bc(k)] = dNa * c - N0 * a * sn * vph;
+          gd[1 + Bs::bs(k)] = -dNa * sn - N0 * a * c * vph;
+        } else {
+          gd[1 + Bs::bc(k)] = dNa;
+        }
       }
     }
   }
 #pragma unroll
-  for (int i = 0; i < kGamStride; ++i) gam[i] = static_cast<float>(g[i]);
+  for (int i = 0; i < kGamStride; ++i) cc.gdot[hl][i] = static_cast<float>(gd[i]);
 }
 
 // Constants of term k shared by a chunk's histograms (from the slot values slot(s) of its
@@ -438,17 +506,26 @@ __device__ __forceinline__ float tile_phase(double nu, double t_start) {
   return static_cast<float>(x - rint(x));
 }
 
+// Tile-level constants of term k (frequency nu) for a tile starting at bin ts: in FP64, its
+// precession phase at that bin reduced to [-1/2, 1/2] turns; with term 0's, the first bin's time.
+template <class SM>
+__device__ __forceinline__ void tile_consts(int ts, const HistSet& hs, int k, double nu, SM& sm) {
+  const double t_start = (static_cast<double>(ts) - sm.cc.t0) * hs.dt_us;
+  if (k == 0) sm.cc.v.tbase = static_cast<float>(t_start);
+  sm.cc.v.base[k] = sm.cc.v.kinds[k] == kTermTF ? tile_phase(nu, t_start) : 0.0f;
+}
+
 // ---------------------------------------------------------------------------------------------
-// Chunk cache fill (only when a CTA moves to another chunk or job).
+// Chunk cache fill (only when a CTA moves to another chunk or job): header, rows, slot values.
 // ---------------------------------------------------------------------------------------------
-template <int SHAPE, class SM>
-__device__ void load_chunk(const Job& job, const HistSet& hs, int job_index, int chunk_index, int prec,
-                           SM& sm) {
-  using Bs = Basis<SHAPE>;
+template <class SM>
+__device__ void load_chunk(const Job& job, const HistSet& hs, int job_index, int chunk_index, SM& sm) {
   ChunkCache& cc = sm.cc;
   const int tid = threadIdx.x;
+  const int nsl = hs.nslots;
+  if (!dbg_ok(job.dbg, chunk_index >= 0 && chunk_index < hs.nchunks, kDbgChunk)) chunk_index = 0;
   if (tid == 0) {
-    const Chunk ch = hs.chunks[dbg_ok(job.dbg, chunk_index >= 0 && chunk_index < hs.nchunks, kDbgChunk) ? chunk_index : 0];
+    const Chunk ch = hs.chunks[chunk_index];
     cc.job = job_index;
     cc.chunk = chunk_index;
     cc.nh = ch.nh;
@@ -461,14 +538,18 @@ __device__ void load_chunk(const Job& job, const HistSet& hs, int job_index, int
     cc.first = ch.first;
     cc.t0 = ch.t0;
   }
-  __syncthreads();
-  const int nh = cc.nh, nsl = hs.nslots;
-  for (int i = tid; i < nh * nsl; i += kBlock) {
+  const bool by_chunk = hs.slot_src != nullptr;  // beside the header, not after it
+  if (!by_chunk) __syncthreads();
+  const int n = (by_chunk ? min(kGroupMax, hs.group) : cc.nh) * nsl;
+  for (int i = tid; i < n; i += kBlock) {
     const int hl = i / nsl, s = i - hl * nsl;
-    int h = hs.hist_index[cc.first + hl];
+    int h = by_chunk ? hs.chunk_hist[chunk_index * kGroupMax + hl] : hs.hist_index[cc.first + hl];
+    if (by_chunk && h < 0) continue;  // beyond the chunk's histograms
     if (!dbg_ok(job.dbg, h >= 0 && h < hs.H, kDbgHist)) h = 0;
-    cc.loc[hl][s] = slot_value(hs, job.params, h, s, job.dbg);
-    const int mi = hs.map[static_cast<int64_t>(h) * hs.nslots + s];
+    const int mi = by_chunk ? hs.slot_src[(chunk_index * kGroupMax + hl) * nsl + s]
+                            : hs.map[static_cast<int64_t>(h) * nsl + s];
+    const bool ok = dbg_ok(job.dbg, mi >= 0 ? mi < hs.P : -1 - mi < hs.nconsts, kDbgMap);
+    cc.loc[hl][s] = !ok ? 0.0 : (mi >= 0 ? job.params[mi] : hs.consts[-1 - mi]);
     cc.ldir[hl][s] = job.dir && mi >= 0 ? job.dir[mi] : 0.0;
     if (s == 0) {
       cc.row[hl] = h;
@@ -479,50 +560,24 @@ __device__ void load_chunk(const Job& job, const HistSet& hs, int job_index, int
     }
   }
   __syncthreads();
-  if (prec == 0) return;
+}
+
+// ... and the SPLIT basis kernels' coefficients and constants of the chunk, with those of its tile
+// (or piece) starting at bin ts (load_tile_at).
+template <int SHAPE, bool GN, class SM>
+__device__ void load_chunk_split(const Job& job, const HistSet& hs, int ts, SM& sm) {
+  using Bs = Basis<SHAPE>;
+  ChunkCache& cc = sm.cc;
+  const int tid = threadIdx.x, nh = cc.nh;
   const double dt = hs.dt_us;
-  if (tid < nh) {
-    const int hl = tid;
-    coef_row<SHAPE>(hs, [&](int q) { return cc.loc[hl][q]; }, cc.v.gam[hl], cc.cph[hl], cc.sph[hl]);
-    const double N0 = cc.loc[hl][0];
-    // Directional derivative of the coefficients along a Gauss-Newton direction (zeros without).
-    double gd[kGamStride];
-#pragma unroll
-    for (int i = 0; i < kGamStride; ++i) gd[i] = 0.0;
-    if (job.dir) {
-      constexpr double kDeg = kTwoPi / 360.0;
-      const double vN0 = cc.ldir[hl][0];
-      gd[0] = cc.ldir[hl][1];
-      gd[1] = hs.envelope ? vN0 : 0.0;
-      if (Bs::MERGED) {
-        const double vph = cc.ldir[hl][hs.canon[0].phi_slot] * kDeg;
-        const double c = cc.cph[hl][0], sn = cc.sph[hl][0];
-        gd[2] = vN0 * c - N0 * sn * vph;
-        gd[3] = -vN0 * sn - N0 * c * vph;
-      } else {
-#pragma unroll
-        for (int k = 0; k < Bs::NT; ++k) {
-          if (k >= hs.nterms) break;
-          const CanonTerm& ct = hs.canon[k];
-          const double a = ct.amp_slot >= 0 ? cc.loc[hl][ct.amp_slot] : 1.0;
-          const double va = ct.amp_slot >= 0 ? cc.ldir[hl][ct.amp_slot] : 0.0;
-          const double dNa = vN0 * a + N0 * va;  // d(N0 a) along v
-          if (ct.kind == kTermTF) {
-            const double vph = cc.ldir[hl][ct.phi_slot] * kDeg;
-            const double c = cc.cph[hl][k], sn = cc.sph[hl][k];
-            gd[1 + Bs::bc(k)] = dNa * c - N0 * a * sn * vph;
-            gd[1 + Bs::bs(k)] = -dNa * sn - N0 * a * c * vph;
-          } else {
-            gd[1 + Bs::bc(k)] = dNa;
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < kGamStride; ++i) cc.gdot[hl][i] = static_cast<float>(gd[i]);
+  if (tid < kGroupMax * kMaxTerms) {  // a lane per (histogram, term)
+    const int hl = tid / kMaxTerms, k = tid - hl * kMaxTerms;
+    if (hl < nh) coef_term<SHAPE>(hs, [&](int q) { return cc.loc[hl][q]; }, k, cc.v.gam[hl], cc.cph[hl], cc.sph[hl]);
   } else if (tid >= 32 && tid < 32 + kMaxTerms) {
     const int k = tid - 32;
-    cc.nu[k] = term_consts(hs, [&](int q) { return cc.loc[0][q]; }, k, cc.v);
+    const double nu = term_consts(hs, [&](int q) { return cc.loc[0][q]; }, k, cc.v);
+    cc.nu[k] = nu;
+    tile_consts(ts, hs, k, nu, sm);
     int src = -1;
     if (k < hs.nterms && hs.canon[k].kind == kTermDKT) {  // the chunk's histograms share (Delta, nu)
       const CanonTerm& ct = hs.canon[k];
@@ -530,7 +585,7 @@ __device__ void load_chunk(const Job& job, const HistSet& hs, int job_index, int
       if (!dbg_ok(job.dbg, src >= 0 && src < hs.ndkt, kDbgDkt)) src = -1;
     }
     cc.v.dkt_src[k] = src;
-    if (k < hs.nterms) {  // directional derivatives of the term's shared parameters (Gauss-Newton products)
+    if (GN && k < hs.nterms) {  // directional derivatives of the term's shared parameters (Gauss-Newton products)
       const CanonTerm& ct = hs.canon[k];
       double dl = 0.0, ds = 0.0;
       for (int i = 0; i < ct.nexp; ++i) dl += cc.ldir[0][ct.exp_slot[i]];
@@ -548,27 +603,23 @@ __device__ void load_chunk(const Job& job, const HistSet& hs, int job_index, int
     // log2(e) / tau_mu: E = 2^(-aE t); without the decay envelope E = 1
     cc.v.aE = hs.envelope ? static_cast<float>(1.4426950408889634 / kTauMuUs) : 0.0f;
     cc.v.dt = static_cast<float>(dt);
+  } else if (tid == 65) {
+    sm.ts.tile_start = ts;
+  }
+  if (GN) {  // the coefficients' directional derivatives need the phases
+    __syncthreads();
+    if (tid < nh) gdot_row<SHAPE>(job, hs, tid, cc);
   }
   __syncthreads();
 }
 
-// Tile-level constants for a tile (or piece) starting at bin ts: its first bin time and, in
-// FP64, each precession phase at that bin reduced to [-1/2, 1/2] turns.
+// A tile (or piece) of the current chunk starting at bin ts.
 template <class SM>
 __device__ void load_tile_at(int ts, const HistSet& hs, int prec, SM& sm) {
   const int tid = threadIdx.x;
   if (tid == 0) sm.ts.tile_start = ts;
-  if (prec == 1 && tid >= 32 && tid < 32 + kMaxTerms) {
-    const int k = tid - 32;
-    const double t_start = (static_cast<double>(ts) - sm.cc.t0) * hs.dt_us;
-    if (k == 0) sm.cc.v.tbase = static_cast<float>(t_start);
-    sm.cc.v.base[k] = sm.cc.v.kinds[k] == kTermTF ? tile_phase(sm.cc.nu[k], t_start) : 0.0f;
-  }
+  if (prec == 1 && tid >= 32 && tid < 32 + kMaxTerms) tile_consts(ts, hs, tid - 32, sm.cc.nu[tid - 32], sm);
   __syncthreads();
-}
-template <class SM>
-__device__ void load_tile(const HistSet& hs, int tile, int prec, SM& sm) {
-  load_tile_at(sm.cc.tile0 + tile * hs.tile_bins, hs, prec, sm);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1047,8 +1098,45 @@ __device__ void list_item(const Job& job, const HistSet& hs, int item, Smem& sm)
 // V_m = sum_j u_j Gam_jm that carry the shared time parameters' derivatives.
 // ---------------------------------------------------------------------------------------------
 // vc: the job's constants on this chunk and tile.
+//
+// FP32 counts are staged into shared memory one iteration ahead by 16-byte cp.async copies, each
+// pair of lanes copying the 4 bins it reads of every histogram (half the histograms each) and
+// meeting at a warp barrier: no CTA-wide barrier per iteration, the warps run independently
+// through the tile.  Borrowed rows are 16-byte aligned with a stride of a multiple of 4, and tiles
+// start at multiples of 4 bins, so every copy is aligned.  stage_counts copies iteration itn of the
+// tile at bin ts into buffer itn & 1: lanes 2q and 2q + 1 of a warp share the block of bins
+// [4q, 4q + 4), the even lane copies it for the even histograms and the odd lane for the odd.
+template <int G>
+__device__ __forceinline__ void stage_counts(const Job& job, const HistSet& hs, Smem& sm, int ts, int iters, int itn) {
+  if (hs.store != kStoreF32) return;
+  const ChunkCache& cc = sm.cc;
+  if (itn < iters) {
+    const int par = threadIdx.x & 1, q4 = (threadIdx.x >> 1) * 4, nh = cc.nh;
+    // n is a multiple of 4 and so is the stride, so n < stride means all 4 bins lie in the row
+    const int64_t n = ts + static_cast<int64_t>(itn) * (kBlock * kBinsPerThread) + q4;
+    const bool in = n < hs.stride;
+#pragma unroll
+    for (int i = 0; i < (G + 1) / 2; ++i) {
+      const int hl = 2 * i + par;
+      if (hl >= nh) break;
+      const bool ok = dbg_ok(job.dbg, cc.row[hl] >= 0 && cc.row[hl] < hs.H && n >= 0, kDbgHist);
+      cp_async16(sm.stage_slot(itn & 1, hl, q4), static_cast<const float*>(cc.rowp[hl]) + (in && ok ? n : 0),
+                 in && ok ? 16u : 0u);
+    }
+  }
+  cp_async_commit();  // one group per iteration (empty past the tile's end)
+}
+
+// Iterations of a tile that hold any bin of the fit range (the same for every thread).
+__device__ __forceinline__ int tile_iterations(int nhi, int ts, int tile_bins) {
+  constexpr int bins = kBlock * kBinsPerThread;
+  return min(tile_bins / bins, (nhi - ts + bins - 1) / bins);
+}
+
+// nit: the CTA iterations of the tile or piece; the counts of the first are already on their way
+// (stage_counts).
 template <int SHAPE, int MODE, bool GRAD>
-__device__ void split_item(const Job& job, const HistSet& hs, int item, Smem& sm, const VecConst& vc, int nit = -1) {
+__device__ void split_item(const Job& job, const HistSet& hs, int item, Smem& sm, const VecConst& vc, int iters) {
   using Bs = Basis<SHAPE>;
   constexpr int NT = Bs::NT;
   constexpr int M = Bs::M;
@@ -1081,36 +1169,8 @@ __device__ void split_item(const Job& job, const HistSet& hs, int item, Smem& sm
     for (int q = 0; q < 4; ++q) sh[k][q] = 0.0f;
 
   constexpr int CHUNK_BINS = kBlock * BPT;  // bins of one CTA iteration
-  // Iterations of this tile that hold any bin of the fit range (the same for every thread);
-  // a piece of a launch-level partition brings its own count.
-  const int iters = nit >= 0 ? nit : min(hs.tile_bins / CHUNK_BINS, (nhi - ts + CHUNK_BINS - 1) / CHUNK_BINS);
-  // FP32 counts are staged into shared memory one iteration ahead by 16-byte cp.async copies,
-  // each pair of lanes copying the 4 bins it reads of every histogram (half the histograms
-  // each) and meeting at a warp barrier: no CTA-wide barrier per iteration, the warps run
-  // independently through the tile.  Borrowed rows are 16-byte aligned with a stride of a
-  // multiple of 4, and tiles start at multiples of 4 bins, so every copy is aligned.
   const bool staged = store == kStoreF32;
   const int64_t stride = hs.stride;
-  // Lanes 2q and 2q + 1 of a warp share the 16-byte block of bins [4q, 4q + 4) of the
-  // iteration: the even lane copies it for the even histograms, the odd lane for the odd.
-  const int par = tb & 1, q4 = (tb >> 1) * 4;
-  auto issue = [&](int itn) {  // bins [4q, 4q + 4) of iteration itn into buffer itn & 1
-    if (itn < iters) {
-      // n is a multiple of 4 and so is stride, so n < stride means all 4 bins lie in the row
-      const int64_t n = ts + static_cast<int64_t>(itn) * CHUNK_BINS + q4;
-      const bool in = n < stride;
-#pragma unroll
-      for (int i = 0; i < (G + 1) / 2; ++i) {
-        const int hl = 2 * i + par;
-        if (hl >= nh) break;
-        const bool ok = dbg_ok(job.dbg, cc.row[hl] >= 0 && cc.row[hl] < hs.H && n >= 0, kDbgHist);
-        cp_async16(sm.stage_slot(itn & 1, hl, q4),
-                   static_cast<const float*>(cc.rowp[hl]) + (in && ok ? n : 0), in && ok ? 16u : 0u);
-      }
-    }
-    cp_async_commit();  // one group per iteration (empty past the tile's end)
-  };
-  if (staged) issue(0);
   // The bin offset in the tile is carried as an exact float (integers < 2^24): an
   // int-to-float conversion per bin would occupy this GPU's slow FP64/conversion pipe.
   float fm0 = static_cast<float>(tb * BPT);
@@ -1123,7 +1183,7 @@ __device__ void split_item(const Job& job, const HistSet& hs, int item, Smem& sm
       // are past it, refill it for it + 1, then wait for this lane's copies of iteration it
       // (all but the newest group) and for the partner's
       __syncwarp();
-      issue(it + 1);
+      stage_counts<G>(job, hs, sm, ts, iters, it + 1);
       cp_async_wait<1>();
       __syncwarp();
     }
@@ -1460,35 +1520,44 @@ __device__ void split_item(const Job& job, const HistSet& hs, int item, Smem& sm
     sm.vred[w][1] = vl;
   }
   if (GRAD) {
+    constexpr int NCHP = (NCH + 31) / 32 * 32;
+    float ch[NCHP];
+#pragma unroll
+    for (int i = NCH; i < NCHP; ++i) ch[i] = 0.0f;
 #pragma unroll
     for (int hl = 0; hl < G; ++hl)
 #pragma unroll
-      for (int q = 0; q < NPH; ++q) {
-        const float r = warp_sum_f(gacc[hl][q]);
-        if (lane == 0) sm.cred[w][hl * NPH + q] = r;
-      }
+      for (int q = 0; q < NPH; ++q) ch[hl * NPH + q] = gacc[hl][q];
 #pragma unroll
     for (int k = 0; k < NT; ++k)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float r = warp_sum_f(sh[k][q]);
-        if (lane == 0) sm.cred[w][G * NPH + k * 4 + q] = r;
-      }
+      for (int q = 0; q < 4; ++q) ch[G * NPH + k * 4 + q] = sh[k][q];
+    warp_scatter_sum<NCHP>(ch);
+#pragma unroll
+    for (int i = 0; i < NCHP / 32; ++i) sm.cred[w][lane * (NCHP / 32) + i] = ch[i];
   }
   __syncthreads();
   static_assert(kWarps == 8, "the FP64 trees below sum 8 warps");
   if (!dbg_ok(job.dbg, item >= 0 && item < job.nrows, kDbgPartial)) return;
   double* row = job.partials + static_cast<int64_t>(item) * hs.pstride;
-  if (GRAD && tid < NCH) {
-    double a[kWarps];
-#pragma unroll
-    for (int i = 0; i < kWarps; ++i) a[i] = static_cast<double>(sm.cred[i][tid]);
-    row[1 + tid] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+  // A channel's eight warps in two halves, on warps 0-1 and 2-3 (one per sub-partition: an FP64
+  // instruction holds its sub-partition for 64 clocks), joined through shared memory.
+  static_assert(NCH <= 64, "a channel per thread of two warps");
+  const int ch = tid & 63, half = tid >> 6;
+  double part = 0.0;
+  if (GRAD && half < 2 && ch < NCH) {
+    const float* c4 = &sm.cred[4 * half][ch];
+    part = (widen(c4[0]) + widen(c4[kMaxChan])) + (widen(c4[2 * kMaxChan]) + widen(c4[3 * kMaxChan]));
+    if (half == 1) (&sm.dred[0][0])[ch] = part;
+  }
+  if (GRAD) {
+    __syncthreads();
+    if (half == 0 && ch < NCH) row[1 + ch] = part + (&sm.dred[0][0])[ch];
   }
   if (tid >= kBlock - 32) {  // the last warp: one lane per warp's float-float value, FP64 tree
     static_assert(NCH <= kBlock - 32, "value warp overlaps a channel thread");
     const int l = tid - (kBlock - 32);
-    double a = l < kWarps ? static_cast<double>(sm.vred[l][0]) + static_cast<double>(sm.vred[l][1]) : 0.0;
+    double a = l < kWarps ? widen(sm.vred[l][0]) + widen(sm.vred[l][1]) : 0.0;
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     // +inf: the likelihood is undefined (N <= 0 where d > 0) or the parameters were not finite.
@@ -1506,9 +1575,8 @@ __device__ double split_slot(const HistSet& hs, const ChunkCache& cc, const doub
   const double N0 = cc.loc[hl][0];
   constexpr double kDeg = kTwoPi / 360.0;
   double g = 0.0;
-  for (int e = 0; e < hs.ncontrib; ++e) {
-    const Contrib c = hs.contrib[e];
-    if (c.slot != s) continue;
+  for (int e = hs.slot_ptr[s]; e < hs.slot_ptr[s + 1]; ++e) {
+    const Contrib c = hs.contrib[hs.slot_list[e]];
     const int k = c.term;
     const CanonTerm& ct = hs.canon[k];
     switch (c.kind) {
@@ -1578,6 +1646,25 @@ __device__ double split_slot(const HistSet& hs, const ChunkCache& cc, const doub
 // ---------------------------------------------------------------------------------------------
 // Completion: chunk finalize, then job finalize.
 // ---------------------------------------------------------------------------------------------
+// Whether a job's columns and its parameters' lists of columns go through shared memory: one chunk,
+// one thread per entry.
+__device__ __forceinline__ bool lists_in_shared(const HistSet& hs) {
+  return hs.nchunks == 1 && hs.P < kBlock && hs.ncols <= kBlock;
+}
+
+// The columns [from, from + unused) of a row that a chunk of nh histograms does not use (basis
+// kernels: the channels of the histograms nh .. G).
+template <int PREC, int SHAPE>
+__device__ __forceinline__ int unused_from(int nh) {
+  if constexpr (PREC == 0 || is_list(SHAPE)) return 1 << 20;
+  return 1 + nh * Basis<SHAPE>::NPH;
+}
+template <int PREC, int SHAPE>
+__device__ __forceinline__ int unused_columns(int nh) {
+  if constexpr (PREC == 0 || is_list(SHAPE)) return 0;
+  return (Basis<SHAPE>::G - nh) * Basis<SHAPE>::NPH;
+}
+
 template <int PREC, int SHAPE, bool GRAD, class SM>
 __device__ void chunk_finalize(const Job& job, const HistSet& hs, SM& sm) {
   const ChunkCache& cc = sm.cc;
@@ -1595,38 +1682,73 @@ __device__ void chunk_finalize(const Job& job, const HistSet& hs, SM& sm) {
   // value-only kernel sums the value column in the same order)
   const int tpc = max(1, min(kBlock / (1 + hs.nch), cc.ntiles));  // threads (segments) per column
   double* seg = reinterpret_cast<double*>(&sm.stage[0][0][0]);  // [nout][tpc], idle staging space
-  if (tid < nout * tpc) {
-    const int c = tid / tpc, k = tid - c * tpc;
-    const int t0 = static_cast<int>(static_cast<int64_t>(cc.ntiles) * k / tpc);
-    const int t1 = static_cast<int>(static_cast<int64_t>(cc.ntiles) * (k + 1) / tpc);
+  // a job of one chunk: the lists of its parameters' columns, on their way while the rows are summed
+  const bool single = GRAD && lists_in_shared(hs);
+  const int first_unused = unused_from<PREC, SHAPE>(cc.nh);
+  int pp = 0, pc = 0;
+  if (single && tid <= hs.P) pp = hs.p_ptr[tid];
+  if (single && tid < hs.ncols) pc = hs.p_cols[tid];
+  // the columns in use: the basis kernels' rows hold zeros for the histograms beyond the chunk's
+  const int skip = first_unused < nout ? unused_columns<PREC, SHAPE>(cc.nh) : 0, ncol = nout - skip;
+  if (tid < ncol * tpc) {
+    const int k = tid / ncol, j = tid - k * ncol;  // neighbouring threads read neighbouring columns
+    const int c = j < first_unused ? j : j + skip;
+    const int t0 = static_cast<int>(static_cast<unsigned>(cc.ntiles) * k / static_cast<unsigned>(tpc));
+    const int t1 = static_cast<int>(static_cast<unsigned>(cc.ntiles) * (k + 1) / static_cast<unsigned>(tpc));
     double a = 0.0;
-    for (int t = t0; t < t1; t += 8) {  // eight rows' loads in flight, added in row order
-      double x[8];
+    for (int t = t0; t < t1; t += 16) {  // sixteen rows' loads in flight, added in row order
+      double x[16];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) x[q] = t + q < t1 ? __ldcg(part + static_cast<int64_t>(t + q) * ps + c) : 0.0;
+      for (int q = 0; q < 16; ++q) x[q] = t + q < t1 ? __ldcg(part + static_cast<int64_t>(t + q) * ps + c) : 0.0;
+      // the full groups as they are, the rest by branches: an addition that is only predicated off
+      // still takes its 64 clocks of the FP64 pipe
 #pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (t + q < t1) a += x[q];
+      for (int q = 0; q < 16; q += 4) {
+        if (t + q + 4 <= t1) {
+          a += x[q];
+          a += x[q + 1];
+          a += x[q + 2];
+          a += x[q + 3];
+        } else {
+          if (t + q >= t1) break;
+          a += x[q];
+          if (t + q + 1 >= t1) break;
+          a += x[q + 1];
+          if (t + q + 2 >= t1) break;
+          a += x[q + 2];
+          break;
+        }
+      }
     }
     seg[c * tpc + k] = a;
+  }
+  if (single) {
+    sm.fin.p_ptr[tid] = pp;
+    sm.fin.p_cols[tid] = pc;
   }
   __syncthreads();
   if (tid < nout) {
     double a = 0.0;
-    for (int k = 0; k < tpc; ++k) a += seg[tid * tpc + k];
+    if (tid < first_unused || tid >= first_unused + skip)
+      for (int k = 0; k < tpc; ++k) a += seg[tid * tpc + k];
     sm.tot[tid] = a;
   }
   __syncthreads();
   if (GRAD) {
     const int nsl = hs.nslots;
-    for (int i = tid; i < cc.nh * nsl; i += kBlock) {
-      const int hl = i / nsl, s = i - hl * nsl;
+    // a warp per slot: its lanes (the histograms) share the slot's formulas, and the slots are spread
+    // over the sub-partitions
+    const int hl = tid & 31;
+    for (int s = tid >> 5; s < nsl && hl < cc.nh; s += kWarps) {
       double g;
       if constexpr (PREC == 0 || is_list(SHAPE))
         g = fp64_slot(hs, sm.tot, s);
       else
         g = split_slot<SHAPE>(hs, cc, sm.tot, hl, s);
-      job.colsum[cc.col0 + i] = g;
+      if (single)
+        sm.fin.cols[cc.col0 + hl * nsl + s] = g;
+      else
+        job.colsum[cc.col0 + hl * nsl + s] = g;
     }
   }
   if (tid == 0) {
@@ -1638,25 +1760,32 @@ __device__ void chunk_finalize(const Job& job, const HistSet& hs, SM& sm) {
 template <class SM>
 __device__ void job_finalize(const Job& job, const HistSet& hs, SM& sm) {
   const int tid = threadIdx.x;
-  double v = 0.0;
-  for (int c = tid; c < hs.nchunks; c += kBlock) v += __ldcg(job.chunk_val + c);
-  v = warp_sum_d(v);
-  if ((tid & 31) == 0) sm.wsum[tid >> 5] = v;
-  __syncthreads();
+  const bool single = lists_in_shared(hs);
   double value = 0.0;
+  if (hs.nchunks == 1) {
+    value = sm.tot[0];
+  } else {
+    double v = 0.0;
+    for (int c = tid; c < hs.nchunks; c += kBlock) v += __ldcg(job.chunk_val + c);
+    v = warp_sum_d(v);
+    if ((tid & 31) == 0) sm.fin.wsum[tid >> 5] = v;
+    __syncthreads();
 #pragma unroll
-  for (int i = 0; i < kWarps; ++i) value += sm.wsum[i];
+    for (int i = 0; i < kWarps; ++i) value += sm.fin.wsum[i];
+  }
   const bool finite = isfinite(value);
   if (job.grad) {
     for (int p = tid; p < hs.P; p += kBlock) {
       double g = 0.0;
-      const int j1 = hs.p_ptr[p + 1];
-      for (int j = hs.p_ptr[p]; j < j1; j += 8) {  // eight loads in flight, summed in column order
+      const int j1 = single ? sm.fin.p_ptr[p + 1] : hs.p_ptr[p + 1];
+      for (int j = single ? sm.fin.p_ptr[p] : hs.p_ptr[p]; j < j1; j += 8) {  // eight loads in flight, summed in order
         double x[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          const int col = j + q < j1 ? hs.p_cols[j + q] : 0;
-          x[q] = j + q < j1 && dbg_ok(job.dbg, col >= 0 && col < hs.ncols, kDbgCol) ? __ldcg(job.colsum + col) : 0.0;
+          const int col = j + q < j1 ? (single ? sm.fin.p_cols[j + q] : hs.p_cols[j + q]) : 0;
+          x[q] = 0.0;
+          if (j + q < j1 && dbg_ok(job.dbg, col >= 0 && col < hs.ncols, kDbgCol))
+            x[q] = single ? sm.fin.cols[col] : __ldcg(job.colsum + col);
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
@@ -1673,11 +1802,10 @@ __device__ void job_finalize(const Job& job, const HistSet& hs, SM& sm) {
 
 // The chunk of a job whose last row has just been published: the CTA sums the chunk's rows
 // (chunk finalize) and, if that chunk was the job's last, the job's chunks (job finalize).
-// Acquire: every thread fences after the acquire-release counter increment that found the
-// chunk complete.
+// Acquire: thread 0's acquire-release increment of the counter that found the chunk complete,
+// and the barrier after it; the rows and sums of other CTAs are read through the L2 (__ldcg).
 template <int PREC, int SHAPE, bool GRAD, class SM>
 __device__ void finish_chunk(const Job& job, const HistSet& hs, SM& sm) {
-  fence_acq_rel();
   chunk_finalize<PREC, SHAPE, GRAD>(job, hs, sm);
   __syncthreads();
   if (hs.nchunks == 1) {  // the chunk was the job's only one: no second counter
@@ -1691,7 +1819,6 @@ __device__ void finish_chunk(const Job& job, const HistSet& hs, SM& sm) {
   }
   __syncthreads();
   if (!sm.flag) return;
-  fence_acq_rel();
   job_finalize(job, hs, sm);
   __syncthreads();
 }
@@ -1700,7 +1827,7 @@ __device__ void finish_chunk(const Job& job, const HistSet& hs, SM& sm) {
 // chunk, and the one that completes a job's last chunk finalizes the job.  Release: the
 // CTA barrier orders every thread's row writes before thread 0's acquire-release counter
 // increment (cumulative over what the barrier ordered before it); acquire: that same
-// atomic, and a fence by every thread of the finalizing CTA.
+// atomic and the barrier behind it.
 template <int PREC, int SHAPE, bool GRAD, class SM>
 __device__ void complete_item(const Job& job, const HistSet& hs, SM& sm) {
   __syncthreads();
@@ -1715,79 +1842,147 @@ __device__ void complete_item(const Job& job, const HistSet& hs, SM& sm) {
 
 // ---------------------------------------------------------------------------------------------
 // Persistent kernel: each CTA takes a contiguous range of the launch's items.
+//
+// A single evaluation is latency: one CTA iteration of work between chains of dependent loads
+// (job, histogram set, item, chunk, histogram, map entry, parameter) at the start and the sums of
+// the rows at the end.  The chain is kept short: the first job comes with the launch, the histogram
+// set goes to shared memory in one step beside the item's entry, and a chunk's map entries stand in
+// a table by chunk.  The FP64 pipe holds a sub-partition for 64 clocks per warp instruction, whatever
+// its lanes do, so set-up, reduction and finalisation are cut into short chains on many warps, and
+// additions of columns known to be 0 are left out.
+// Measured (GB300, cycles from the kernel's start to the job's end in the last CTA): 8 x 65536 bins
+// 31500 -> 26000, 1 x 16384 bins 24700 -> 18500; calls with their host side 44.5 -> 32.7 us and
+// 36.0 -> 27.0 us (with the parameters in the launch and the results written to host memory), a fit
+// of the former 517 -> 385 us, 16 x 81920 bins at 64 vectors (chi^2) 129.7 -> 118.6 us, 64 x 2^20 at
+// 64 (-2lnL) 6.90 -> 6.70 ms.
 // ---------------------------------------------------------------------------------------------
+
+// Makes job ji and its histogram set current (shared memory).  All threads; barriers inside.
+template <class SM>
+__device__ void enter_job(const LaunchHead& head, int ji, SM& sm) {
+  __syncthreads();  // the job before is no longer read
+  const int tid = threadIdx.x;
+  const HistSet* src = ji == 0 ? head.first.hs : head.jobs[ji].hs;
+  if (ji == 0) {
+    if (tid < static_cast<int>(sizeof(Job) / 8))
+      reinterpret_cast<uint64_t*>(&sm.job)[tid] = reinterpret_cast<const uint64_t*>(&head.first)[tid];
+  } else {
+    static_assert(sizeof(Job) % 8 == 0 && sizeof(Job) / 8 <= kBlock, "a job in one step");
+    if (tid < static_cast<int>(sizeof(Job) / 8))
+      reinterpret_cast<uint64_t*>(&sm.job)[tid] = reinterpret_cast<const uint64_t*>(head.jobs + ji)[tid];
+  }
+  if (ji == 0 && head.nx > 0 && tid < head.nx) sm.x[tid] = head.x[tid];
+  if (sm.hs_src != src) {
+    static_assert(sizeof(HistSet) % 16 == 0 && sizeof(HistSet) / 16 <= kBlock, "a histogram set in one step");
+    if (tid < static_cast<int>(sizeof(HistSet) / 16))
+      reinterpret_cast<int4*>(&sm.hs)[tid] = reinterpret_cast<const int4*>(src)[tid];
+  }
+  __syncthreads();
+  if (tid == 0) sm.hs_src = src;  // read again only after another barrier
+  if (ji == 0 && head.nx > 0) {
+    if (tid == 0) sm.job.params = sm.x;
+    __syncthreads();
+  }
+}
+
+// The job of global item gi: by division where every job has per_job items, else the last job whose
+// first item is not after gi (counted by the whole CTA, in one round of loads per kBlock jobs).
+__device__ __forceinline__ int job_of_item(const LaunchHead& head, int gi) {
+  if (head.per_job > 0) return gi / head.per_job;
+  int n = 0;
+  for (int j = threadIdx.x; j - static_cast<int>(threadIdx.x) < head.njobs; j += kBlock)
+    n += __syncthreads_count(j < head.njobs && head.jobs[j].item_begin <= gi);
+  return n > 0 ? n - 1 : 0;
+}
+
 template <int PREC, int SHAPE, int MODE, bool GRAD>
 __global__ void __launch_bounds__(kBlock, PREC == 1 && SHAPE != kShapeList ? 2 : 1) eval_kernel(
-    const Job* __restrict__ jobs, int njobs,
-                                                      int total_items) {
+    const __grid_constant__ LaunchHead head) {
   __shared__ Smem sm;
-  const int per = (total_items + gridDim.x - 1) / gridDim.x;
+  const int per = (head.total_items + gridDim.x - 1) / gridDim.x;
   const int beg = blockIdx.x * per;
-  const int end = min(total_items, beg + per);
+  const int end = min(head.total_items, beg + per);
   if (threadIdx.x == 0) {
     sm.cc.job = -1;
     sm.cc.chunk = -1;
+    sm.hs_src = nullptr;
   }
-  __syncthreads();
+  const Job& job = sm.job;
+  const HistSet& hs = sm.hs;
+  int ji = -1;
   if constexpr (PREC == 1 && !is_list(SHAPE)) {
-    if (jobs[0].pieces) {  // launch-level partition: this CTA's pieces, in order
-      if (static_cast<int>(blockIdx.x) >= jobs[0].npiece_ctas) return;
-      const int pb = jobs[0].piece_cta[blockIdx.x], pe = jobs[0].piece_cta[blockIdx.x + 1];
+    if (head.first.pieces) {  // launch-level partition: this CTA's pieces, in order
+      if (static_cast<int>(blockIdx.x) >= head.first.npiece_ctas) return;
+      const int pb = head.first.piece_cta[blockIdx.x], pe = head.first.piece_cta[blockIdx.x + 1];
       for (int p = pb; p < pe; ++p) {
-        const Piece pc = jobs[0].pieces[p];
-        if (!dbg_ok(jobs[0].dbg, pc.job >= 0 && pc.job < njobs, kDbgJob)) continue;
-        const Job job = jobs[pc.job];
-        const HistSet& hs = *job.hs;
-        if (sm.cc.job != pc.job || sm.cc.chunk != pc.chunk) {
+        const Piece pc = head.first.pieces[p];
+        if (!dbg_ok(head.first.dbg, pc.job >= 0 && pc.job < head.njobs, kDbgJob)) continue;
+        if (pc.job != ji) {
+          ji = pc.job;
+          enter_job(head, ji, sm);
+        }
+        const bool fresh = sm.cc.job != pc.job || sm.cc.chunk != pc.chunk;
+        if (fresh) {
           __syncthreads();
-          load_chunk<SHAPE>(job, hs, pc.job, pc.chunk, PREC, sm);
-          if (threadIdx.x == 0) {  // the chunk's rows in this partition (load_tile_at's barrier publishes them)
+          load_chunk(job, hs, pc.job, pc.chunk, sm);
+        }
+        const int ts = sm.cc.tile0 + pc.it0 * (kBlock * kBinsPerThread);
+        stage_counts<Basis<SHAPE>::G>(job, hs, sm, ts, pc.nit, 0);
+        if (fresh) {
+          load_chunk_split<SHAPE, MODE == 2 || MODE == 3>(job, hs, ts, sm);
+          if (threadIdx.x == 0) {  // the chunk's rows in this partition (read after the item's barriers)
             const int2 r = job.chunk_rows[pc.chunk];
             sm.cc.item0 = r.x;
             sm.cc.ntiles = r.y;
           }
+        } else {
+          load_tile_at(ts, hs, PREC, sm);
         }
-        load_tile_at(sm.cc.tile0 + pc.it0 * (kBlock * kBinsPerThread), hs, PREC, sm);
         split_item<SHAPE, MODE, GRAD>(job, hs, pc.row, sm, sm.cc.v, pc.nit);
         complete_item<PREC, SHAPE, GRAD>(job, hs, sm);
       }
       return;
     }
   }
-  int ji = -1;
-  Job job;
+  if (beg >= end) return;
   for (int gi = beg; gi < end; ++gi) {
-    if (ji < 0 || gi >= job.item_begin + job.hs->nitems) {
-      int lo = 0, hi = njobs - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (jobs[mid].item_begin <= gi)
-          lo = mid;
-        else
-          hi = mid - 1;
-      }
-      ji = lo;
-      job = jobs[ji];
+    int chunk = -1;
+    if (ji < 0) {
+      ji = job_of_item(head, gi);
+      if (ji == 0) chunk = head.first.items[gi].x;  // on its way beside the histogram set
+      enter_job(head, ji, sm);
     }
-    const HistSet& hs = *job.hs;
+    while (gi >= job.item_begin + hs.nitems) {  // jobs without items are passed over
+      enter_job(head, ++ji, sm);
+      chunk = -1;
+    }
     const int item = gi - job.item_begin;
-    // term lists without a basis form take the FP64 path's chunk and tile setup
-    constexpr int kSetupPrec = is_list(SHAPE) ? 0 : PREC;
-    if (sm.cc.job != ji || item < sm.cc.item0 || item >= sm.cc.item0 + sm.cc.ntiles) {
+    const bool fresh = sm.cc.job != ji || item < sm.cc.item0 || item >= sm.cc.item0 + sm.cc.ntiles;
+    if (fresh) {
+      if (chunk < 0) chunk = job.items[item].x;
       __syncthreads();
-      load_chunk<SHAPE>(job, hs, ji, hs.items[item].x, kSetupPrec, sm);
-      if constexpr (PREC == 1 && is_list(SHAPE)) load_chunk_list(hs, sm);
+      load_chunk(job, hs, ji, chunk, sm);
     }
-    load_tile(hs, item - sm.cc.item0, kSetupPrec, sm);
-    if constexpr (PREC == 1 && is_list(SHAPE)) load_tile_list(hs, sm);
-    if constexpr (PREC == 0)
-      fp64_item<MODE, GRAD>(job, hs, item, sm);
-    else if constexpr (SHAPE == kShapeList)
-      list_item<MODE, GRAD, kMaxTerms, kMaxPrims>(job, hs, item, sm);
-    else if constexpr (SHAPE == kShapeListS)  // at most 2 terms of at most 3 primitives
-      list_item<MODE, GRAD, 2, 3>(job, hs, item, sm);
-    else
-      split_item<SHAPE, MODE, GRAD>(job, hs, item, sm, sm.cc.v);
+    const int ts = sm.cc.tile0 + (item - sm.cc.item0) * hs.tile_bins;
+    if constexpr (PREC == 1 && !is_list(SHAPE)) {
+      const int iters = tile_iterations(sm.cc.nhi, ts, hs.tile_bins);
+      stage_counts<Basis<SHAPE>::G>(job, hs, sm, ts, iters, 0);
+      if (fresh)
+        load_chunk_split<SHAPE, MODE == 2 || MODE == 3>(job, hs, ts, sm);
+      else
+        load_tile_at(ts, hs, PREC, sm);
+      split_item<SHAPE, MODE, GRAD>(job, hs, item, sm, sm.cc.v, iters);
+    } else {  // term lists, on the FP64 path or per bin in FP32
+      if (PREC == 1 && fresh) load_chunk_list(hs, sm);
+      load_tile_at(ts, hs, 0, sm);
+      if (PREC == 1) load_tile_list(hs, sm);
+      if constexpr (PREC == 0)
+        fp64_item<MODE, GRAD>(job, hs, item, sm);
+      else if constexpr (SHAPE == kShapeList)
+        list_item<MODE, GRAD, kMaxTerms, kMaxPrims>(job, hs, item, sm);
+      else  // at most 2 terms of at most 3 primitives
+        list_item<MODE, GRAD, 2, 3>(job, hs, item, sm);
+    }
     complete_item<PREC, SHAPE, GRAD>(job, hs, sm);
   }
 }
@@ -1807,16 +2002,15 @@ int resident_ctas() {
 }
 
 template <int PREC, int SHAPE, int MODE, bool GRAD>
-int launch_one(const Job* d_jobs, int njobs, int total_items, int num_sms, cudaStream_t stream,
-               LaunchInfo* info) {
+int launch_one(const LaunchHead& head, int num_sms, cudaStream_t stream, LaunchInfo* info) {
   auto kern = eval_kernel<PREC, SHAPE, MODE, GRAD>;
   int per_sm = resident_ctas<PREC, SHAPE, MODE, GRAD>();
   if (per_sm < 0) return -1;
   if (per_sm < 1) per_sm = 1;
   int grid = num_sms * per_sm;
-  if (grid > total_items) grid = total_items;
+  if (grid > head.total_items) grid = head.total_items;
   if (grid < 1) grid = 1;
-  kern<<<grid, kBlock, 0, stream>>>(d_jobs, njobs, total_items);
+  kern<<<grid, kBlock, 0, stream>>>(head);
   if (info) {
     info->grid = grid;
     info->block = kBlock;
@@ -1831,22 +2025,21 @@ int occupancy_one() {
 }
 
 template <int PREC, int SHAPE>
-int dispatch_mode(int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
-                  LaunchInfo* info) {
+int dispatch_mode(int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s, LaunchInfo* info) {
   if constexpr (is_list(SHAPE)) {  // no Gauss-Newton kernels for term lists (FP64 path)
     if (mode == 2 || mode == 3) return -1;
   } else {
-    if (mode == 2) return launch_one<PREC, SHAPE, 2, true>(j, n, items, sms, s, info);
-    if (mode == 3) return launch_one<PREC, SHAPE, 3, true>(j, n, items, sms, s, info);
+    if (mode == 2) return launch_one<PREC, SHAPE, 2, true>(h, sms, s, info);
+    if (mode == 3) return launch_one<PREC, SHAPE, 3, true>(h, sms, s, info);
   }
   if (PREC == 1 && mode == 4)  // weighted chi^2 of asymmetry data (SPLIT)
-    return grad ? launch_one<PREC, SHAPE, PREC == 1 ? 4 : 0, true>(j, n, items, sms, s, info)
-                : launch_one<PREC, SHAPE, PREC == 1 ? 4 : 0, false>(j, n, items, sms, s, info);
+    return grad ? launch_one<PREC, SHAPE, PREC == 1 ? 4 : 0, true>(h, sms, s, info)
+                : launch_one<PREC, SHAPE, PREC == 1 ? 4 : 0, false>(h, sms, s, info);
   if (mode == 0)
-    return grad ? launch_one<PREC, SHAPE, 0, true>(j, n, items, sms, s, info)
-                : launch_one<PREC, SHAPE, 0, false>(j, n, items, sms, s, info);
-  return grad ? launch_one<PREC, SHAPE, 1, true>(j, n, items, sms, s, info)
-              : launch_one<PREC, SHAPE, 1, false>(j, n, items, sms, s, info);
+    return grad ? launch_one<PREC, SHAPE, 0, true>(h, sms, s, info)
+                : launch_one<PREC, SHAPE, 0, false>(h, sms, s, info);
+  return grad ? launch_one<PREC, SHAPE, 1, true>(h, sms, s, info)
+              : launch_one<PREC, SHAPE, 1, false>(h, sms, s, info);
 }
 
 template <int PREC, int SHAPE>
@@ -1868,10 +2061,10 @@ int occupancy_mode(int mode, int grad) {
 }  // namespace kern
 
 // Per-group launchers and occupancy queries (one translation unit each).
-int launch_group_fp64(int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s, LaunchInfo* info);
+int launch_group_fp64(int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s, LaunchInfo* info);
 int occupancy_group_fp64(int mode, int grad);
 #define MUSR_DECLARE_GROUP(G)                                                                                \
-  int launch_group_##G(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s, \
+  int launch_group_##G(int shape, int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s,            \
                        LaunchInfo* info);                                                                   \
   int occupancy_group_##G(int shape, int mode, int grad);
 MUSR_DECLARE_GROUP(a)
@@ -1879,11 +2072,11 @@ MUSR_DECLARE_GROUP(b)
 MUSR_DECLARE_GROUP(c)
 #undef MUSR_DECLARE_GROUP
 // The FP64 basis kernels (musr_kernels_f64.cuh), by the same groups of shapes.
-int launch_group_f64_a(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
+int launch_group_f64_a(int shape, int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s,
                        LaunchInfo* info);
-int launch_group_f64_b(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
+int launch_group_f64_b(int shape, int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s,
                        LaunchInfo* info);
-int launch_group_f64_c(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
+int launch_group_f64_c(int shape, int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s,
                        LaunchInfo* info);
 
 }  // namespace musr

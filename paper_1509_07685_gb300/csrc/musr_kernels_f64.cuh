@@ -54,12 +54,16 @@ struct Chunk64 {
 struct Smem64 {
   // idle staging space of chunk_finalize ([columns][segments] doubles, at most kBlock of them)
   alignas(16) float stage[1][1][2 * kBlock];
+  Job job;
+  double x[kHeadParams];
+  HistSet hs;
+  const HistSet* hs_src;
   ChunkCache cc;
   TileState ts;
+  Finish fin;
   Chunk64 c;
   double red[kWarps][64];
   double tot[kMaxChan + 1];
-  double wsum[kWarps];
   double2 logtab[kLogTable];  // (c, -ln c) per interval
   int flag;
 };
@@ -67,16 +71,6 @@ struct Smem64 {
 // ---------------------------------------------------------------------------------------------
 // Arithmetic
 // ---------------------------------------------------------------------------------------------
-
-// A float as a double on the integer pipe (a conversion instruction would occupy the FP64
-// pipe); subnormal floats, which counts never are, take the conversion.
-__device__ __forceinline__ double widen(float f) {
-  const unsigned b = __float_as_uint(f);
-  const unsigned e = b & 0x7f800000u;
-  if (e == 0u && (b & 0x007fffffu)) return static_cast<double>(f);
-  const unsigned hi = (b & 0x80000000u) | (e ? ((b & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
-  return __hiloint2double(static_cast<int>(hi), static_cast<int>(b << 29));
-}
 
 // Whether x > 0 and x > 1 (x not a NaN): doubles order like their bits for positive values.
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
@@ -115,34 +109,36 @@ __device__ __forceinline__ double ln_tab(double x, const double2* tab) {
   return l;
 }
 
-// The table: c = 1 / (midpoint of the interval), rounded to FP32, and -ln c of that c.
-__device__ __forceinline__ void fill_log_table(double2* tab) {
-  static_assert(kLogTable == kBlock, "one interval per thread");
-  const int lo = kLogOff + (static_cast<int>(threadIdx.x) << 12);
-  const double mid = 0.5 * (__hiloint2double(lo, 0) + __hiloint2double(lo + 0x1000, 0));
-  // the interval that begins at 1 takes c = 1: ln is then exactly 0 at x = 1
-  const double c = lo == 0x3ff00000 ? 1.0 : static_cast<double>(static_cast<float>(1.0 / mid));
-  tab[threadIdx.x] = make_double2(c, -log(c));
+// The table, computed when the library is compiled (a logarithm per thread at every launch would
+// cost it 2 us): c = 1 / (midpoint of the interval) in 24 bits or fewer (1 for the interval that
+// begins at 1: ln is then exactly 0 at x = 1), and -ln c of that c by the series of atanh,
+// ln c = 2 (z + z^3/3 + ...), z = (c - 1)/(c + 1), |z| < 0.18, summed from its smallest term.
+struct LogTable {
+  double2 t[kLogTable];
+};
+constexpr double neg_ln(double c) {
+  const double z = (c - 1.0) / (c + 1.0), z2 = z * z;
+  double s = 0.0;
+  for (int k = 25; k >= 3; k -= 2) s = (s + 1.0 / k) * z2;
+  return -2.0 * (z + z * s);
 }
-
-// Sums a[0 .. N) over the warp's lanes, N a multiple of 32: a lane keeps N / 32 of the sums (lane
-// l the entries l N / 32 ..., in a[0 .. N / 32)).  Each step adds half of what is left, N - N / 32
-// FP64 additions per warp where a butterfly per entry takes 5 N; every entry is summed in the
-// order of warp_sum_d.
-template <int N>
-__device__ __forceinline__ void warp_scatter_sum(double (&a)[N]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 16, n = N / 2; o > 0; o >>= 1, n >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < N / 2; ++i) {
-      if (i >= n) break;
-      const double keep = up ? a[i + n] : a[i], send = up ? a[i] : a[i + n];
-      a[i] = __dadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, o));
-    }
+constexpr LogTable make_log_table() {
+  LogTable r{};
+  for (int i = 0; i < kLogTable; ++i) {
+    // high words from 0x3fe6a000 in steps of 0x1000: mantissa 1 + w / 2^20, below 1 at half the scale
+    const int lo = kLogOff + (i << 12), up = lo + 0x1000;
+    auto value = [](int hi) {
+      const double m = 1.0 + (hi & 0xfffff) / 1048576.0;
+      return (hi >> 20) == 0x3ff ? m : 0.5 * m;
+    };
+    const double mid = 0.5 * (value(lo) + value(up));
+    const double c = lo == 0x3ff00000 ? 1.0 : static_cast<double>(static_cast<float>(1.0 / mid));
+    r.t[i].x = c;
+    r.t[i].y = lo == 0x3ff00000 ? 0.0 : neg_ln(c);
   }
+  return r;
 }
+__device__ const LogTable log_table = make_log_table();
 
 // ---------------------------------------------------------------------------------------------
 // Chunk set-up
@@ -246,7 +242,8 @@ __device__ void load_chunk64(const Job& job, const HistSet& hs, Smem64& sm) {
   // beside the coefficients of the histograms.
   static_assert(kRebase == 32 && kWarps > kMaxTerms + 1, "one lane per table entry");
   const int wp = tid >> 5, i = tid & 31;
-  if (wp >= 2 && wp < 2 + kMaxTerms) {
+  const bool many = hs.tile_bins > kBlock;  // an item of one iteration needs no table
+  if (many && wp >= 2 && wp < 2 + kMaxTerms) {
     const int k = wp - 2;
     if (k < hs.nterms && k < Bs::NT) {
       const double ti = i * D, z = c.kt[k] * ti;
@@ -260,7 +257,7 @@ __device__ void load_chunk64(const Job& job, const HistSet& hs, Smem64& sm) {
       if (c.kinds[k] == kTermKT || c.kinds[k] == kTermLKT)
         c.qk[k][i] = exp(c.kinds[k] == kTermKT ? -(0.5 * z * z) : -z);
     }
-  } else if (wp == 2 + kMaxTerms) {
+  } else if (many && wp == 2 + kMaxTerms) {
     c.qe[i] = exp(-c.rate * (i * D));
   }
   if (tid < nh) {
@@ -367,7 +364,7 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
         if (k >= nterms) continue;
         const double S = c.S[k];
         fc[k] = __dmul_rn(c.bamp[k], exp(-__dmul_rn(__fma_rn(__dmul_rn(0.5, S), t, c.lam[k]), t)));
-        if (S != 0.0) w[k] = exp(-__dmul_rn(__dmul_rn(S, t), kBlock * dt));
+        if (S != 0.0 && iters > 1) w[k] = exp(-__dmul_rn(__dmul_rn(S, t), kBlock * dt));
         if (Bs::tf(c.kinds, k)) {
           const double p = __dmul_rn(c.st_hi[k], nd);  // phase in turns, as a double-double
           const double pl = __fma_rn(c.st_lo[k], nd, __fma_rn(c.st_hi[k], nd, -p));
@@ -378,7 +375,7 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
         } else if (c.kinds[k] == kTermKT) {
           const double z = __dmul_rn(c.kt[k], t);
           fk[k] = exp(-__dmul_rn(__dmul_rn(0.5, z), z));
-          wk[k] = exp(-__dmul_rn(__dmul_rn(__dmul_rn(c.kt[k], c.kt[k]), t), kBlock * dt));
+          if (iters > 1) wk[k] = exp(-__dmul_rn(__dmul_rn(__dmul_rn(c.kt[k], c.kt[k]), t), kBlock * dt));
         } else if (c.kinds[k] == kTermLKT) {
           fk[k] = exp(-__dmul_rn(c.kt[k], t));
         }
@@ -608,49 +605,48 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
 // The first of these executes 47 FP64 instructions per pair (16 of them fresh time factors, a CTA
 // having two iterations), the second 33, the third 31.
 template <int SHAPE, int MODE, bool GRAD>
-__global__ void __launch_bounds__(kBlock, 1) eval64_kernel(const Job* __restrict__ jobs, int njobs, int total_items) {
+__global__ void __launch_bounds__(kBlock, 1) eval64_kernel(const __grid_constant__ LaunchHead head) {
   __shared__ Smem64 sm;
-  const int per = (total_items + gridDim.x - 1) / gridDim.x;
-  const int beg = blockIdx.x * per, end = min(total_items, beg + per);
+  const int per = (head.total_items + gridDim.x - 1) / gridDim.x;
+  const int beg = blockIdx.x * per, end = min(head.total_items, beg + per);
   if (threadIdx.x == 0) {
     sm.cc.job = -1;
     sm.cc.chunk = -1;
+    sm.hs_src = nullptr;
   }
-  if (MODE == 1) fill_log_table(sm.logtab);
-  __syncthreads();
+  if (MODE == 1) sm.logtab[threadIdx.x] = log_table.t[threadIdx.x];  // read after several barriers
+  const Job& job = sm.job;
+  const HistSet& hs = sm.hs;
   int ji = -1;
-  Job job;
   for (int gi = beg; gi < end; ++gi) {
-    if (ji < 0 || gi >= job.item_begin + job.hs->nitems) {
-      int lo = 0, hi = njobs - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (jobs[mid].item_begin <= gi)
-          lo = mid;
-        else
-          hi = mid - 1;
-      }
-      ji = lo;
-      job = jobs[ji];
+    int chunk = -1;
+    if (ji < 0) {
+      ji = job_of_item(head, gi);
+      if (ji == 0) chunk = head.first.items[gi].x;  // on its way beside the histogram set
+      enter_job(head, ji, sm);
     }
-    const HistSet& hs = *job.hs;
+    while (gi >= job.item_begin + hs.nitems) {
+      enter_job(head, ++ji, sm);
+      chunk = -1;
+    }
     const int item = gi - job.item_begin;
     if (sm.cc.job != ji || item < sm.cc.item0 || item >= sm.cc.item0 + sm.cc.ntiles) {
+      if (chunk < 0) chunk = job.items[item].x;
       __syncthreads();
-      load_chunk<SHAPE>(job, hs, ji, hs.items[item].x, 0, sm);
+      load_chunk(job, hs, ji, chunk, sm);
       load_chunk64<SHAPE>(job, hs, sm);
     }
-    load_tile(hs, item - sm.cc.item0, 0, sm);
+    load_tile_at(sm.cc.tile0 + (item - sm.cc.item0) * hs.tile_bins, hs, 0, sm);
     basis64_item<SHAPE, MODE, GRAD>(job, hs, item, sm);
     complete_item<2, SHAPE, GRAD>(job, hs, sm);
   }
 }
 
 template <int SHAPE, int MODE, bool GRAD>
-int launch64(const Job* d_jobs, int njobs, int total_items, int num_sms, cudaStream_t stream, LaunchInfo* info) {
-  int grid = num_sms < total_items ? num_sms : total_items;
+int launch64(const LaunchHead& head, int num_sms, cudaStream_t stream, LaunchInfo* info) {
+  int grid = num_sms < head.total_items ? num_sms : head.total_items;
   if (grid < 1) grid = 1;
-  eval64_kernel<SHAPE, MODE, GRAD><<<grid, kBlock, 0, stream>>>(d_jobs, njobs, total_items);
+  eval64_kernel<SHAPE, MODE, GRAD><<<grid, kBlock, 0, stream>>>(head);
   if (info) {
     info->grid = grid;
     info->block = kBlock;
@@ -659,12 +655,11 @@ int launch64(const Job* d_jobs, int njobs, int total_items, int num_sms, cudaStr
 }
 
 template <int SHAPE>
-int dispatch64(int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s, LaunchInfo* info) {
-  if (mode == 2) return launch64<SHAPE, 2, true>(j, n, items, sms, s, info);
-  if (mode == 3) return launch64<SHAPE, 3, true>(j, n, items, sms, s, info);
-  if (mode == 0)
-    return grad ? launch64<SHAPE, 0, true>(j, n, items, sms, s, info) : launch64<SHAPE, 0, false>(j, n, items, sms, s, info);
-  return grad ? launch64<SHAPE, 1, true>(j, n, items, sms, s, info) : launch64<SHAPE, 1, false>(j, n, items, sms, s, info);
+int dispatch64(int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s, LaunchInfo* info) {
+  if (mode == 2) return launch64<SHAPE, 2, true>(h, sms, s, info);
+  if (mode == 3) return launch64<SHAPE, 3, true>(h, sms, s, info);
+  if (mode == 0) return grad ? launch64<SHAPE, 0, true>(h, sms, s, info) : launch64<SHAPE, 0, false>(h, sms, s, info);
+  return grad ? launch64<SHAPE, 1, true>(h, sms, s, info) : launch64<SHAPE, 1, false>(h, sms, s, info);
 }
 
 }  // namespace

@@ -3,17 +3,17 @@
 
 namespace musr {
 
-int launch_group_f64_a(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
+int launch_group_f64_a(int shape, int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s,
                        LaunchInfo* info) {
   switch (shape) {
     case kShapeGeneric:
-      return kern::dispatch64<kShapeGeneric>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch64<kShapeGeneric>(mode, grad, h, sms, s, info);
     case kShapeT1:
-      return kern::dispatch64<kShapeT1>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch64<kShapeT1>(mode, grad, h, sms, s, info);
     case kShapeN1:
-      return kern::dispatch64<kShapeN1>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch64<kShapeN1>(mode, grad, h, sms, s, info);
     case kShapeT1N1:
-      return kern::dispatch64<kShapeT1N1>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch64<kShapeT1N1>(mode, grad, h, sms, s, info);
     default:
       return -1;
   }

@@ -3,8 +3,8 @@
 
 namespace musr {
 
-int launch_group_fp64(int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s, LaunchInfo* info) {
-  return kern::dispatch_mode<0, 0>(mode, grad, j, n, items, sms, s, info);
+int launch_group_fp64(int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s, LaunchInfo* info) {
+  return kern::dispatch_mode<0, 0>(mode, grad, h, sms, s, info);
 }
 int occupancy_group_fp64(int mode, int grad) { return kern::occupancy_mode<0, 0>(mode, grad); }
 

@@ -3,21 +3,20 @@
 
 namespace musr {
 
-int launch_group_a(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
-                     LaunchInfo* info) {
+int launch_group_a(int shape, int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s, LaunchInfo* info) {
   switch (shape) {
     case kShapeGeneric:
-      return kern::dispatch_mode<1, kShapeGeneric>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch_mode<1, kShapeGeneric>(mode, grad, h, sms, s, info);
     case kShapeT1:
-      return kern::dispatch_mode<1, kShapeT1>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch_mode<1, kShapeT1>(mode, grad, h, sms, s, info);
     case kShapeN1:
-      return kern::dispatch_mode<1, kShapeN1>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch_mode<1, kShapeN1>(mode, grad, h, sms, s, info);
     case kShapeT1N1:
-      return kern::dispatch_mode<1, kShapeT1N1>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch_mode<1, kShapeT1N1>(mode, grad, h, sms, s, info);
     case kShapeList:
-      return kern::dispatch_mode<1, kShapeList>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch_mode<1, kShapeList>(mode, grad, h, sms, s, info);
     case kShapeListS:
-      return kern::dispatch_mode<1, kShapeListS>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch_mode<1, kShapeListS>(mode, grad, h, sms, s, info);
     default:
       return -1;
   }

@@ -3,13 +3,12 @@
 
 namespace musr {
 
-int launch_group_c(int shape, int mode, int grad, const Job* j, int n, int items, int sms, cudaStream_t s,
-                     LaunchInfo* info) {
+int launch_group_c(int shape, int mode, int grad, const LaunchHead& h, int sms, cudaStream_t s, LaunchInfo* info) {
   switch (shape) {
     case kShapeT2m:
-      return kern::dispatch_mode<1, kShapeT2m>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch_mode<1, kShapeT2m>(mode, grad, h, sms, s, info);
     case kShapeT2N1m:
-      return kern::dispatch_mode<1, kShapeT2N1m>(mode, grad, j, n, items, sms, s, info);
+      return kern::dispatch_mode<1, kShapeT2N1m>(mode, grad, h, sms, s, info);
     default:
       return -1;
   }

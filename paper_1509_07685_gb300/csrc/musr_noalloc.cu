@@ -341,6 +341,7 @@ extern "C" int musr_eval_noalloc(const void* d_counts, int dtype, int nhist, int
   job.hs = &dT->hs;
   job.params = d_params;
   job.out = d_out;
+  job.items = dT->items;
   job.partials = d_part;
   job.nrows = nitems;
   job.colsum = d_cols;
@@ -359,7 +360,8 @@ extern "C" int musr_eval_noalloc(const void* d_counts, int dtype, int nhist, int
   e = cudaMemsetAsync(d_zero, 0, sizeof(unsigned) * (nchunks + 1), stream);
   if (e != cudaSuccess) return na_cuda(e, "cudaMemsetAsync(counters)");
   LaunchInfo info;
-  if (launch_eval(precision, hs.shape, mode, job.grad, &dT->job, 1, nitems, num_sms, cuda_stream, &info))
+  const LaunchHead head{&dT->job, 1, nitems, nitems, 0, job, {}};
+  if (launch_eval(precision, hs.shape, mode, job.grad, head, num_sms, cuda_stream, &info))
     return na_cuda(cudaGetLastError(), "kernel launch");
   return MUSR_OK;
 }

@@ -181,6 +181,13 @@ inline const char* plan_split(const musr_term* terms, int nterms, const int32_t*
       if (!merged || k == 0) add(ct.phi_slot, kCPhi, k);
     }
   }
+  int n = 0;
+  for (int s = 0; s < kMaxSlots; ++s) {
+    hs->slot_ptr[s] = static_cast<unsigned char>(n);
+    for (int e = 0; e < hs->ncontrib; ++e)
+      if (hs->contrib[e].slot == s) hs->slot_list[n++] = static_cast<unsigned char>(e);
+  }
+  hs->slot_ptr[kMaxSlots] = static_cast<unsigned char>(n);
   return nullptr;
 }
 

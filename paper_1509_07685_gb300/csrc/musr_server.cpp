@@ -534,8 +534,8 @@ int launch_lane(musr_server* s, int L) {
   for (const Launch& Lc : launches) {
     if (Lc.items == 0) continue;
     LaunchInfo info;
-    if (launch_eval(Lc.prec, Lc.shape, Lc.mode, 1, d_jobs + Lc.first, Lc.njobs, Lc.items, s->num_sms, s->stream,
-                    &info))
+    const LaunchHead head{d_jobs + Lc.first, Lc.njobs, Lc.items, 0, 0, lane.h_jobs[Lc.first], {}};
+    if (launch_eval(Lc.prec, Lc.shape, Lc.mode, 1, head, s->num_sms, s->stream, &info))
       return MUSR_ECUDA;
   }
   e = cudaMemcpyAsync(lane.h_out, d_out, no * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
