@@ -990,6 +990,7 @@ void musr_ctx_destroy(musr_ctx* ctx) {
   dfree(ctx, ev.counters);
   dfree(ctx, ev.jobs);
   dfree(ctx, ev.dirs);
+  dfree(ctx, ev.gram);
   dfree(ctx, ev.dkt);
   dfree(ctx, ev.dkt_work);
   dfree(ctx, ev.dkt_count);
@@ -1450,11 +1451,80 @@ int musr_gn_product(musr_ctx* ctx, const double* params, int nparams, const doub
   return MUSR_OK;
 }
 
+// The FP64 matrix in one pass (musr_gram64.cu) for theories with a basis form and at most 12 fitted
+// local slots.  Returns 1 when this call is not of that kind (nothing enqueued): the products then
+// answer it, and report whatever is wrong with it.
+static int gram_matrix(musr_ctx* ctx, const double* params, int mode, double* out) {
+  if (check_ready(ctx, mode, MUSR_FP64) || !params) return 1;
+  const int P = ctx->P;
+  for (int i = 0; i < P; ++i)
+    if (!std::isfinite(params[i])) return 1;
+  const int var = pick_variant(ctx, MUSR_FP64, 1);
+  const HistSet& hs = ctx->comp[MUSR_FP64][var].hs;
+  if (hs.nitems == 0 || hs.shape == kShapeList || hs.ndkt > 0 || hs.nchunks > 65535) return 1;
+  bool active[musr::kMaxSlots] = {};
+  for (int h = 0; h < ctx->H; ++h)
+    for (int s = 0; s < ctx->nslots; ++s) active[s] |= ctx->map[static_cast<size_t>(h) * ctx->nslots + s] >= 0;
+  musr::GramPlan plan;
+  if (!musr::gram_plan(hs, active, mode + 2, &plan)) return 1;
+  EvalBufs& ev = ctx->ev;
+  const int ne = musr::gram_values(plan.nj);
+  const size_t nsum = static_cast<size_t>(hs.nchunks) * musr::kGroupMax * ne;
+  const size_t rows = static_cast<size_t>(musr::gram_rows(plan, hs.nchunks, ctx->num_sms)) * sizeof(double);
+  if (ev.gram.bytes < rows && dalloc(ctx, ev.gram, rows)) return 1;  // beyond the budget: the products need less
+  const bool in_launch = P <= musr::kHeadParams;
+  if (!in_launch && ev.params.bytes < P * sizeof(double)) return 1;  // its buffer comes with the first evaluation
+  if (ensure_uploaded(ctx, MUSR_FP64, var)) return 1;
+  int rc;
+  if ((rc = ensure_host(ctx, &ev.h_in, &ev.h_in_bytes, P * sizeof(double)))) return rc;
+  if ((rc = ensure_host(ctx, &ev.h_out, &ev.h_out_bytes, nsum * sizeof(double)))) return rc;
+  musr::LaunchHead head{nullptr, 1, hs.nitems, hs.nitems, 0, Job{}, {}};
+  fill_jobs(ctx, MUSR_FP64, var, mode + 2, 1, 1, static_cast<const double*>(ev.params.p), nullptr, &head.first, 0, nullptr);
+  cudaError_t e = cudaSuccess;
+  if (in_launch) {
+    head.nx = P;
+    std::memcpy(head.x, params, sizeof(double) * P);
+  } else {
+    std::memcpy(ev.h_in, params, sizeof(double) * P);
+    e = cudaMemcpyAsync(ev.params.p, ev.h_in, sizeof(double) * P, cudaMemcpyHostToDevice, ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpyAsync(params)");
+  }
+  if (musr::launch_gram(hs.shape, plan, head, hs.nchunks, static_cast<double*>(ev.gram.p), ev.h_out, ctx->num_sms, ctx->stream))
+    return cuda_fail(ctx, cudaGetLastError(), "Gauss-Newton matrix launch");
+  e = cudaStreamSynchronize(ctx->stream);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaStreamSynchronize");
+  // local slots to parameters
+  const Compiled& c = ctx->comp[MUSR_FP64][var];
+  std::vector<double> H(static_cast<size_t>(P) * P, 0.0);
+  bool finite = true;
+  for (int ci = 0; ci < hs.nchunks; ++ci)
+    for (int hl = 0; hl < c.chunks[ci].nh; ++hl) {
+      const double* v = ev.h_out + (static_cast<size_t>(ci) * musr::kGroupMax + hl) * ne;
+      const int32_t* row = ctx->map.data() + static_cast<size_t>(c.hist_index[c.chunks[ci].first + hl]) * ctx->nslots;
+      for (int i = 0; i < plan.nj; ++i)
+        for (int j = 0; j <= i; ++j, ++v) {
+          finite = finite && std::isfinite(*v);
+          const int32_t p = row[plan.slot[i]], q = row[plan.slot[j]];
+          if (p < 0 || q < 0) continue;
+          H[static_cast<size_t>(p) * P + q] += *v;
+          if (i != j) H[static_cast<size_t>(q) * P + p] += *v;
+        }
+    }
+  if (!finite) return fail(ctx, MUSR_ENONFINITE, "-2lnL undefined: N <= 0 in a bin with d > 0, or a parameter not finite");
+  std::memcpy(out, H.data(), sizeof(double) * H.size());
+  return MUSR_OK;
+}
+
 int musr_gauss_newton(musr_ctx* ctx, const double* params, int nparams, int mode, int precision, double* out) {
   if (!ctx) return MUSR_EINVAL;
   if (!out) return fail(ctx, MUSR_EINVAL, "out must not be NULL");
   if (nparams != ctx->P || nparams < 1) return fail(ctx, MUSR_EINVAL, "nparams does not match the map");
   const size_t P = nparams;
+  if (precision == MUSR_FP64) {
+    DeviceScope ds(ctx->device);
+    const int rc = gram_matrix(ctx, params, mode, out);
+    if (rc <= 0) return rc;
+  }
   std::vector<double> dirs(P * P, 0.0), prod(P * (P + 1));
   for (size_t i = 0; i < P; ++i) dirs[i * P + i] = 1.0;
   const int rc = musr_gn_product(ctx, params, nparams, dirs.data(), nparams, mode, precision, prod.data());

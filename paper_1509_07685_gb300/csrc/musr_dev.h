@@ -266,6 +266,35 @@ struct LaunchHead {
 };
 
 // Launchers (host side of musr_kernels.cu).  All enqueue on `stream`.
+// The Gauss-Newton matrix of a basis theory in one pass (musr_gram64.cu): the local slots j < nj
+// (slot 0, N0, first) and the derivative of N by each as a sum over entries [ptr[j], ptr[j + 1]) of a
+// coefficient per histogram times a function of time.
+constexpr int kGramSlots = 12, kGramEntries = 56;
+enum GramCoef : unsigned char {  // a: amplitude, c, s: cosine and sine of the phase, G: a coefficient Gam
+  kGOne, kGN0C, kGN0S, kGN0P,          // 1; by N0: a c, -a s, a
+  kGAmpC, kGAmpS, kGAmpP,              // by a: N0 c, -N0 s, N0
+  kGPhiC, kGPhiS,                      // by phi (degrees): -N0 a s, -N0 a c
+  kGLamC, kGLamS, kGSigC, kGSigS,      // by a rate: -G; by a width sigma: -sigma G
+  kGNuC, kGNuS,                        // by a frequency: 2 pi G_s, -2 pi G_c
+  kGDel, kGLkt, kGDkt                  // by Delta: (2/3) Delta G, (2/3) G, G
+};
+struct GramEntry {
+  unsigned char func, coef, term, slot;  // func 255: the constant 1
+};
+struct GramPlan {
+  int nj, mode;  // mode 2: chi^2, 3: -2lnL
+  unsigned char slot[kGramSlots], ptr[kGramSlots + 1];
+  GramEntry e[kGramEntries];
+};
+inline int gram_values(int nj) { return nj <= 8 ? 36 : 78; }  // of the kernel's triangle (row by row)
+// The plan for the slots with active[s]; false if they or their entries are too many.
+bool gram_plan(const HistSet& hs, const bool* active, int mode, GramPlan* plan);
+// Enqueues the matrix's parts of every histogram: sums [nchunks][kGroupMax][gram_values(nj)] (device-visible),
+// rows: scratch of gram_rows() doubles.
+int64_t gram_rows(const GramPlan& plan, int nchunks, int num_sms);
+int launch_gram(int shape, const GramPlan& plan, const LaunchHead& head, int nchunks, double* rows, double* sums,
+                int num_sms, void* stream);
+
 struct LaunchInfo {
   int grid;
   int block;

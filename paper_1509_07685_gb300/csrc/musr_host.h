@@ -72,6 +72,7 @@ struct EvalBufs {
   DevBuf params, out, partials, colsum, chunk_val, chunk_count, counters, jobs, dirs;
   DevBuf dkt, dkt_work;  // dynamic Kubo-Toyabe tables and their solve's scratch, per evaluation
   DevBuf dkt_count;      // their completion counters (zeroed once; each solve adds 2)
+  DevBuf gram;           // rows of a Gauss-Newton matrix
   DevBuf part;           // a launch-level partition: chunk rows, CTA offsets, pieces
   double* h_in = nullptr;
   double* h_out = nullptr;

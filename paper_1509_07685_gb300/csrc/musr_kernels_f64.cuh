@@ -176,8 +176,8 @@ __device__ void dcoef_row64(const HistSet& hs, Slot slot, Dir dir, const double*
 }
 
 // After load_chunk (header, slot values, row pointers): the FP64 coefficients and constants.
-template <int SHAPE>
-__device__ void load_chunk64(const Job& job, const HistSet& hs, Smem64& sm) {
+template <int SHAPE, class SM>
+__device__ void load_chunk64(const Job& job, const HistSet& hs, SM& sm) {
   using Bs = Basis<SHAPE>;
   ChunkCache& cc = sm.cc;
   Chunk64& c = sm.c;
@@ -312,6 +312,107 @@ __device__ void load_chunk64(const Job& job, const HistSet& hs, Smem64& sm) {
   __syncthreads();
 }
 
+// A thread's time factors, its bins kBlock apart.  at() gives the pieces of the bin at time t (nd bins
+// from time zero), `step` steps after the last bin evaluated afresh (0: evaluates this one; the steps
+// are taken in order, and many says whether any follow): the envelope E, per term P with its cosine
+// and sine parts, and a Kubo-Toyabe term's derivative factors dK (along Delta) and, in Ps, dynamic
+// Kubo-Toyabe's along nu.
+template <int SHAPE>
+struct TimeFactors {
+  using Bs = Basis<SHAPE>;
+  static constexpr int NT = Bs::NT;
+  // Per term at the last fresh bin: the factor a exp(-L t - S t^2/2) with its cosine and sine
+  // parts (fc, fs), a Gaussian's cross ratio of one step w (already in fc, fs for the steps made),
+  // and the same of a Kubo-Toyabe term's own exponential (fk, wk); the envelope (fE).
+  double fE, fc[NT], fs[NT], w[NT], fk[NT], wk[NT];
+
+  __device__ __forceinline__ TimeFactors() {
+    fE = 0.0;
+#pragma unroll
+    for (int k = 0; k < NT; ++k) fc[k] = fs[k] = fk[k] = 0.0, w[k] = wk[k] = 1.0;
+  }
+
+  __device__ __forceinline__ void at(const Job& job, const HistSet& hs, const Chunk64& c, int step, bool many, double nd,
+                                     double t, double* E, double (&Pc)[NT], double (&Ps)[NT], double (&dK)[NT]) {
+    const int nterms = Bs::NTF < 0 ? min(hs.nterms, NT) : NT;
+    if (step == 0) {
+      fE = exp(-__dmul_rn(c.rate, t));
+#pragma unroll
+      for (int k = 0; k < NT; ++k) {
+        if (k >= nterms) continue;
+        const double S = c.S[k];
+        fc[k] = __dmul_rn(c.bamp[k], exp(-__dmul_rn(__fma_rn(__dmul_rn(0.5, S), t, c.lam[k]), t)));
+        if (S != 0.0 && many) w[k] = exp(-__dmul_rn(__dmul_rn(S, t), kBlock * hs.dt_us));
+        if (Bs::tf(c.kinds, k)) {
+          const double p = __dmul_rn(c.st_hi[k], nd);  // phase in turns, as a double-double
+          const double pl = __fma_rn(c.st_lo[k], nd, __fma_rn(c.st_hi[k], nd, -p));
+          double s, co;
+          sincospi(__dmul_rn(2.0, __dadd_rn(__dadd_rn(p, -rint(p)), pl)), &s, &co);
+          fs[k] = __dmul_rn(fc[k], s);
+          fc[k] = __dmul_rn(fc[k], co);
+        } else if (c.kinds[k] == kTermKT) {
+          const double z = __dmul_rn(c.kt[k], t);
+          fk[k] = exp(-__dmul_rn(__dmul_rn(0.5, z), z));
+          if (many) wk[k] = exp(-__dmul_rn(__dmul_rn(__dmul_rn(c.kt[k], c.kt[k]), t), kBlock * hs.dt_us));
+        } else if (c.kinds[k] == kTermLKT) {
+          fk[k] = exp(-__dmul_rn(c.kt[k], t));
+        }
+      }
+    }
+    *E = fE;
+    double xc[NT], xs[NT], kg[NT];
+#pragma unroll
+    for (int k = 0; k < NT; ++k) xc[k] = fc[k], xs[k] = fs[k], kg[k] = fk[k];
+    if (step != 0) {
+      *E = __dmul_rn(fE, c.qe[step]);
+#pragma unroll
+      for (int k = 0; k < NT; ++k) {
+        if (k >= nterms) continue;
+        const double2 q = c.q[k][step];
+        if (c.S[k] != 0.0) fc[k] = __dmul_rn(fc[k], w[k]);
+        if (Bs::tf(c.kinds, k)) {
+          if (c.S[k] != 0.0) fs[k] = __dmul_rn(fs[k], w[k]);
+          xc[k] = __fma_rn(fc[k], q.x, -__dmul_rn(fs[k], q.y));
+          xs[k] = __fma_rn(fc[k], q.y, __dmul_rn(fs[k], q.x));
+        } else {
+          xc[k] = __dmul_rn(fc[k], q.x);
+          if (c.kinds[k] == kTermKT) fk[k] = __dmul_rn(fk[k], wk[k]);
+          if (c.kinds[k] == kTermKT || c.kinds[k] == kTermLKT) kg[k] = __dmul_rn(fk[k], c.qk[k][step]);
+        }
+      }
+    }
+    // Time-only pieces of the bin: P (with cosine and sine parts), and a Kubo-Toyabe term's
+    // derivative factors dK (along Delta) and, in Ps, dynamic Kubo-Toyabe's along nu.
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+      Pc[k] = xc[k];
+      Ps[k] = xs[k];
+      dK[k] = 0.0;
+      if (k >= nterms || Bs::tf(c.kinds, k)) continue;
+      const int kind = c.kinds[k];
+      if (kind == kTermKT) {
+        const double z = __dmul_rn(c.kt[k], t), u = __dmul_rn(z, z);
+        const double Xg = __dmul_rn(xc[k], kg[k]);
+        dK[k] = __dmul_rn(__dmul_rn(Xg, __dmul_rn(t, t)), __dadd_rn(u, -3.0));
+        Pc[k] = __fma_rn(__dmul_rn(2.0 / 3.0, __dadd_rn(1.0, -u)), Xg, __dmul_rn(xc[k], 1.0 / 3.0));
+      } else if (kind == kTermLKT) {
+        const double u = __dmul_rn(c.kt[k], t);
+        const double Xg = __dmul_rn(xc[k], kg[k]);
+        dK[k] = __dmul_rn(__dmul_rn(Xg, t), __dadd_rn(u, -2.0));
+        Pc[k] = __fma_rn(__dmul_rn(2.0 / 3.0, __dadd_rn(1.0, -u)), Xg, __dmul_rn(xc[k], 1.0 / 3.0));
+      } else if (Bs::DKT && kind == kTermDKT) {
+        double Gd = 1.0, gD = 0.0, gN = 0.0;
+        if (c.dkt_src[k] >= 0)
+          dkt_lookup(static_cast<const double*>(job.dkt) + static_cast<size_t>(c.dkt_src[k]) * kDktTable, t, &Gd, &gD,
+                     &gN);
+        dK[k] = __dmul_rn(xc[k], gD);
+        Ps[k] = __dmul_rn(xc[k], gN);
+        Pc[k] = __dmul_rn(xc[k], Gd);
+      }
+    }
+  }
+};
+
 // ---------------------------------------------------------------------------------------------
 // One work item: a tile of one chunk.  Channels, rows and their finalisation as on the SPLIT
 // path (split_item), in FP64.  The cost's value is formed by explicitly rounded operations only,
@@ -344,94 +445,14 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
     for (int q = 0; q < 4; ++q) sh[k][q] = 0.0;
   int bad = 0;
 
-  // Per term at the last fresh bin: the factor a exp(-L t - S t^2/2) with its cosine and sine
-  // parts (fc, fs), a Gaussian's cross ratio of one step w (already in fc, fs for the steps made),
-  // and the same of a Kubo-Toyabe term's own exponential (fk, wk); the envelope (fE).
-  double fE = 0.0, fc[NT], fs[NT], w[NT], fk[NT], wk[NT];
-#pragma unroll
-  for (int k = 0; k < NT; ++k) fc[k] = fs[k] = fk[k] = 0.0, w[k] = wk[k] = 1.0;
-
+  TimeFactors<SHAPE> tf;
   const int iters = min(hs.tile_bins / kBlock, (nhi - ts + kBlock - 1) / kBlock);
   double nd = __dadd_rn(static_cast<double>(ts + tid), -cc.t0);  // bin - t0
   for (int it = 0; it < iters; ++it) {
     const int n = ts + it * kBlock + tid;
     const double t = __dmul_rn(nd, dt);
-    const int step = safe ? it & (kRebase - 1) : 0;  // steps from the last fresh bin
-    if (step == 0) {
-      fE = exp(-__dmul_rn(c.rate, t));
-#pragma unroll
-      for (int k = 0; k < NT; ++k) {
-        if (k >= nterms) continue;
-        const double S = c.S[k];
-        fc[k] = __dmul_rn(c.bamp[k], exp(-__dmul_rn(__fma_rn(__dmul_rn(0.5, S), t, c.lam[k]), t)));
-        if (S != 0.0 && iters > 1) w[k] = exp(-__dmul_rn(__dmul_rn(S, t), kBlock * dt));
-        if (Bs::tf(c.kinds, k)) {
-          const double p = __dmul_rn(c.st_hi[k], nd);  // phase in turns, as a double-double
-          const double pl = __fma_rn(c.st_lo[k], nd, __fma_rn(c.st_hi[k], nd, -p));
-          double s, co;
-          sincospi(__dmul_rn(2.0, __dadd_rn(__dadd_rn(p, -rint(p)), pl)), &s, &co);
-          fs[k] = __dmul_rn(fc[k], s);
-          fc[k] = __dmul_rn(fc[k], co);
-        } else if (c.kinds[k] == kTermKT) {
-          const double z = __dmul_rn(c.kt[k], t);
-          fk[k] = exp(-__dmul_rn(__dmul_rn(0.5, z), z));
-          if (iters > 1) wk[k] = exp(-__dmul_rn(__dmul_rn(__dmul_rn(c.kt[k], c.kt[k]), t), kBlock * dt));
-        } else if (c.kinds[k] == kTermLKT) {
-          fk[k] = exp(-__dmul_rn(c.kt[k], t));
-        }
-      }
-    }
-    double E = fE, xc[NT], xs[NT], kg[NT];
-#pragma unroll
-    for (int k = 0; k < NT; ++k) xc[k] = fc[k], xs[k] = fs[k], kg[k] = fk[k];
-    if (step != 0) {
-      E = __dmul_rn(fE, c.qe[step]);
-#pragma unroll
-      for (int k = 0; k < NT; ++k) {
-        if (k >= nterms) continue;
-        const double2 q = c.q[k][step];
-        if (c.S[k] != 0.0) fc[k] = __dmul_rn(fc[k], w[k]);
-        if (Bs::tf(c.kinds, k)) {
-          if (c.S[k] != 0.0) fs[k] = __dmul_rn(fs[k], w[k]);
-          xc[k] = __fma_rn(fc[k], q.x, -__dmul_rn(fs[k], q.y));
-          xs[k] = __fma_rn(fc[k], q.y, __dmul_rn(fs[k], q.x));
-        } else {
-          xc[k] = __dmul_rn(fc[k], q.x);
-          if (c.kinds[k] == kTermKT) fk[k] = __dmul_rn(fk[k], wk[k]);
-          if (c.kinds[k] == kTermKT || c.kinds[k] == kTermLKT) kg[k] = __dmul_rn(fk[k], c.qk[k][step]);
-        }
-      }
-    }
-    // Time-only pieces of the bin: P (with cosine and sine parts), and a Kubo-Toyabe term's
-    // derivative factors dK (along Delta) and, in Ps, dynamic Kubo-Toyabe's along nu.
-    double Pc[NT], Ps[NT], dK[NT];
-#pragma unroll
-    for (int k = 0; k < NT; ++k) {
-      Pc[k] = xc[k];
-      Ps[k] = xs[k];
-      dK[k] = 0.0;
-      if (k >= nterms || Bs::tf(c.kinds, k)) continue;
-      const int kind = c.kinds[k];
-      if (kind == kTermKT) {
-        const double z = __dmul_rn(c.kt[k], t), u = __dmul_rn(z, z);
-        const double Xg = __dmul_rn(xc[k], kg[k]);
-        dK[k] = __dmul_rn(__dmul_rn(Xg, __dmul_rn(t, t)), __dadd_rn(u, -3.0));
-        Pc[k] = __fma_rn(__dmul_rn(2.0 / 3.0, __dadd_rn(1.0, -u)), Xg, __dmul_rn(xc[k], 1.0 / 3.0));
-      } else if (kind == kTermLKT) {
-        const double u = __dmul_rn(c.kt[k], t);
-        const double Xg = __dmul_rn(xc[k], kg[k]);
-        dK[k] = __dmul_rn(__dmul_rn(Xg, t), __dadd_rn(u, -2.0));
-        Pc[k] = __fma_rn(__dmul_rn(2.0 / 3.0, __dadd_rn(1.0, -u)), Xg, __dmul_rn(xc[k], 1.0 / 3.0));
-      } else if (Bs::DKT && kind == kTermDKT) {
-        double Gd = 1.0, gD = 0.0, gN = 0.0;
-        if (c.dkt_src[k] >= 0)
-          dkt_lookup(static_cast<const double*>(job.dkt) + static_cast<size_t>(c.dkt_src[k]) * kDktTable, t, &Gd, &gD,
-                     &gN);
-        dK[k] = __dmul_rn(xc[k], gD);
-        Ps[k] = __dmul_rn(xc[k], gN);
-        Pc[k] = __dmul_rn(xc[k], Gd);
-      }
-    }
+    double E, Pc[NT], Ps[NT], dK[NT];
+    tf.at(job, hs, c, safe ? it & (kRebase - 1) : 0, iters > 1, nd, t, &E, Pc, Ps, dK);
     double Bf[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) Bf[m] = m == 0 ? E : 0.0;
@@ -599,9 +620,10 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
 // decomposition is picked for that grid.
 // Measured on GB300 (a call with its copies, before: the term-list kernel with CUDA's library
 // functions per histogram and bin):
-//   8 x 65536 bins, two cosine terms, -2lnL value and gradient, one vector   467 ->   93 us
-//   1 x 16384 bins, one cosine term, -2lnL at 1000 vectors                  4116 -> 1154 us
-//   8 x 65536 bins, Gauss-Newton products along 28 directions               8884 ->  853 us
+//   8 x 65536 bins, two cosine terms, -2lnL value and gradient, one vector   467 ->   80 us
+//   1 x 16384 bins, one cosine term, -2lnL at 1000 vectors                  4116 -> 1114 us
+//   8 x 65536 bins, Gauss-Newton products along 28 directions               8884 ->  849 us
+//   (the whole matrix: musr_gram64.cu)
 // The first of these executes 47 FP64 instructions per pair (16 of them fresh time factors, a CTA
 // having two iterations), the second 33, the third 31.
 template <int SHAPE, int MODE, bool GRAD>

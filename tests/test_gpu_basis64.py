@@ -1,7 +1,7 @@
 """The FP64 basis kernels (musr_kernels_f64.cuh) against the oracle where they can go wrong: the
 edges of a CTA iteration (256 bins) and of the bins between two fresh evaluations of the time
 factors (32 iterations), chunks of one to nine histograms, every shape, time zero inside the
-histogram, parameters whose factors under- or overflow (evaluated afresh in every bin), FP64 and
+histogram, the Gauss-Newton matrix in one pass (musr_gram64.cu), parameters whose factors under- or overflow (evaluated afresh in every bin), FP64 and
 FP32 stores.  Tolerance: the FP64 path's, 1e-12 of the value and of each gradient scale."""
 import numpy as np
 import pytest
@@ -63,6 +63,8 @@ def _check(p, x, modes=(0, 1), gn=False):
                 H, ref = ctx.gauss_newton(x, mode, B.MUSR_FP64), oracle.gauss_newton(p, x, mode)
                 d = np.sqrt(np.diag(ref))
                 assert np.all(np.abs(H - ref) <= 1e-12 * np.outer(d, d) + 1e-300)
+                _, prod, _ = ctx.gn_product(x, np.eye(x.size), mode, B.MUSR_FP64)  # the same by products
+                assert np.all(np.abs(H - 0.5 * (prod + prod.T)) <= 1e-12 * np.outer(d, d) + 1e-300)
 
 
 @pytest.mark.parametrize("shape", list(TERMS))
