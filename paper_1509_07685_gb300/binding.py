@@ -148,8 +148,16 @@ def load():
     return _lib
 
 
+_DOUBLES = ctypes.c_double * 1
+
+
 def _dptr(a: np.ndarray):
-    return a.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+    """A contiguous float64 array as a C pointer that keeps the array alive.  Over the array's buffer where it
+    is writable (0.3 us), else through ndarray.ctypes (1.5 us; read-only and empty arrays)."""
+    try:
+        return _DOUBLES.from_buffer(a)
+    except (TypeError, ValueError):
+        return a.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
 
 
 def _err(ctx, status: int):
