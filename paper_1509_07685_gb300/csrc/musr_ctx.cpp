@@ -612,8 +612,8 @@ int pick_variant(musr_ctx* ctx, int prec, int nvec) {
   return musr::pick_decomposition(items, nvec, prec, ctx->num_sms);
 }
 
-// Buffers for nvec evaluations; rebuilds the job table when the launch's key
-// (precision, decomposition, mode, grad, nvec, pointers) changes.
+// Buffers for nvec evaluations (the job table is rebuilt when one of them moves or the launch's
+// key -- precision, decomposition, mode, grad, nvec -- changes; prepare_jobs)
 int ensure_eval(musr_ctx* ctx, int prec, int var, int nvec) {
   EvalBufs& ev = ctx->ev;
   int urc = ensure_uploaded(ctx, prec, var);
@@ -729,8 +729,7 @@ bool plan_partition(musr_ctx* ctx, int prec, int var, int mode, int grad, int nv
   return true;
 }
 
-int prepare_jobs(musr_ctx* ctx, int prec, int var, int mode, int grad, int nvec, const double* d_params,
-                 double* d_out, const double* d_dirs, const Partition* part = nullptr) {
+int prepare_jobs(musr_ctx* ctx, int prec, int var, int mode, int grad, int nvec, const Partition* part = nullptr) {
   EvalBufs& ev = ctx->ev;
   int rc;
   if ((rc = ensure_eval(ctx, prec, var, nvec))) return rc;
@@ -740,11 +739,23 @@ int prepare_jobs(musr_ctx* ctx, int prec, int var, int mode, int grad, int nvec,
   }
   const bool pieces = part != nullptr;
   if (ev.key_valid && ev.k_prec == prec && ev.k_var == var && ev.k_mode == mode && ev.k_grad == grad &&
-      ev.k_nvec == nvec && ev.k_params == d_params && ev.k_out == d_out && ev.k_dirs == d_dirs &&
-      ev.k_pieces == pieces)
+      ev.k_nvec == nvec && ev.k_pieces == pieces)
     return MUSR_OK;
   std::vector<Job> jobs(nvec);
-  fill_jobs(ctx, prec, var, mode, grad, nvec, d_params, d_out, jobs.data(), 0, d_dirs);
+  fill_jobs(ctx, prec, var, mode, grad, nvec, nullptr, nullptr, jobs.data(), 0, nullptr);  // where: LaunchHead.io
+  const bool table = nvec > 1 || ctx->comp[prec][var].hs.ndkt > 0;  // else the launch carries the only job
+  if (!table) {
+    ev.first = jobs[0];
+    ev.key_valid = true;
+    ev.k_prec = prec;
+    ev.k_var = var;
+    ev.k_mode = mode;
+    ev.k_grad = grad;
+    ev.k_nvec = nvec;
+    ev.k_pieces = false;
+    ev.k_grid = 0;
+    return MUSR_OK;
+  }
   cudaError_t e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaStreamSynchronize");
   if (pieces) {  // the partition's rows, tables and the jobs' pointers into them
@@ -789,9 +800,6 @@ int prepare_jobs(musr_ctx* ctx, int prec, int var, int mode, int grad, int nvec,
   ev.k_mode = mode;
   ev.k_grad = grad;
   ev.k_nvec = nvec;
-  ev.k_params = d_params;
-  ev.k_out = d_out;
-  ev.k_dirs = d_dirs;
   ev.k_pieces = pieces;
   ev.k_grid = pieces ? part->grid : 0;
   return MUSR_OK;
@@ -818,6 +826,7 @@ struct LaunchPlan {
   bool empty = false, pieces = false;
   int grid = 0;
   double* d_out = nullptr;
+  musr::LaunchIo io{};
   const double* x = nullptr;  // one evaluation's parameters (host), to go with the launch
 };
 
@@ -835,8 +844,9 @@ int plan_launch(musr_ctx* ctx, int prec, int mode, int grad, int nvec, const dou
   if (L->empty) return MUSR_OK;
   musr::max_ctas_per_sm(prec, hs.shape, mode, grad);  // the occupancy query, before any capture
   const EvalBufs& ev = ctx->ev;
+  L->io = {d_params, d_out, d_dirs, ctx->P};
   if (ev.key_valid && ev.k_prec == prec && ev.k_var == L->var && ev.k_mode == mode && ev.k_grad == grad &&
-      ev.k_nvec == nvec && ev.k_params == d_params && ev.k_out == d_out && ev.k_dirs == d_dirs) {
+      ev.k_nvec == nvec) {
     L->pieces = ev.k_pieces;  // the job table and partition on the device are this launch's
     L->grid = ev.k_grid;
     return MUSR_OK;
@@ -847,7 +857,7 @@ int plan_launch(musr_ctx* ctx, int prec, int mode, int grad, int nvec, const dou
               hs.shape != musr::kShapeList && hs.shape != musr::kShapeListS &&
               plan_partition(ctx, prec, L->var, mode, grad, nvec, &part);
   L->grid = L->pieces ? part.grid : 0;
-  return prepare_jobs(ctx, prec, L->var, mode, grad, nvec, d_params, d_out, d_dirs, L->pieces ? &part : nullptr);
+  return prepare_jobs(ctx, prec, L->var, mode, grad, nvec, L->pieces ? &part : nullptr);
 }
 
 int issue_launch(musr_ctx* ctx, const LaunchPlan& L) {
@@ -858,13 +868,13 @@ int issue_launch(musr_ctx* ctx, const LaunchPlan& L) {
   }
   musr::LaunchInfo info;
   if (hs.ndkt > 0 &&
-      musr::launch_dkt_tables(L.prec, static_cast<const Job*>(ctx->ev.jobs.p), L.nvec, hs.ndkt, ctx->stream)) {
+      musr::launch_dkt_tables(L.prec, static_cast<const Job*>(ctx->ev.jobs.p), L.nvec, hs.ndkt, L.io, ctx->stream)) {
     cudaError_t e = cudaGetLastError();
     ctx->ev.key_valid = false;
     return cuda_fail(ctx, e, "dynamic Kubo-Toyabe table launch");
   }
   musr::LaunchHead head{static_cast<const Job*>(ctx->ev.jobs.p), L.nvec, L.pieces ? L.grid : L.nvec * hs.nitems,
-                        hs.nitems, 0, ctx->ev.first, {}};
+                        hs.nitems, 0, L.io, ctx->ev.first, {}};
   if (L.x) {
     head.nx = ctx->P;
     std::memcpy(head.x, L.x, sizeof(double) * ctx->P);
@@ -1478,7 +1488,7 @@ static int gram_matrix(musr_ctx* ctx, const double* params, int mode, double* ou
   int rc;
   if ((rc = ensure_host(ctx, &ev.h_in, &ev.h_in_bytes, P * sizeof(double)))) return rc;
   if ((rc = ensure_host(ctx, &ev.h_out, &ev.h_out_bytes, nsum * sizeof(double)))) return rc;
-  musr::LaunchHead head{nullptr, 1, hs.nitems, hs.nitems, 0, Job{}, {}};
+  musr::LaunchHead head{nullptr, 1, hs.nitems, hs.nitems, 0, {}, Job{}, {}};
   fill_jobs(ctx, MUSR_FP64, var, mode + 2, 1, 1, static_cast<const double*>(ev.params.p), nullptr, &head.first, 0, nullptr);
   cudaError_t e = cudaSuccess;
   if (in_launch) {

@@ -256,11 +256,20 @@ enum DebugCheck : unsigned {
 // work items (its CTAs with a launch-level partition), the items of every job where the jobs share
 // one histogram set (0: they do not), and the first job itself (a single evaluation reads no job
 // from memory).
-// x: the parameters of a launch of one job that come with it (nx of them; 0: at first.params).
+// x: the parameters of a launch of one job that come with it (nx of them; 0: none).  io: where job j's
+// parameters, results and direction lie, at j P, j (1 + P) and j P (null: in the job itself), so that a
+// caller's new buffers need no new table of jobs.
 constexpr int kHeadParams = 128;
+struct LaunchIo {
+  const double* params;
+  double* out;
+  const double* dirs;
+  int64_t P;
+};
 struct LaunchHead {
   const Job* jobs;
   int njobs, total_items, per_job, nx;
+  LaunchIo io;
   Job first;
   double x[kHeadParams];
 };
@@ -304,7 +313,7 @@ int launch_eval(int precision, int shape, int mode, int grad, const LaunchHead& 
 int max_ctas_per_sm(int precision, int shape, int mode, int grad);
 // The dynamic Kubo-Toyabe tables of njobs evaluations of one histogram set (precision 0:
 // FP64, 1: FP32), two CTAs per (job, source); enqueued on `stream` before the evaluation.
-int launch_dkt_tables(int precision, const Job* d_jobs, int njobs, int ndkt, void* stream);
+int launch_dkt_tables(int precision, const Job* d_jobs, int njobs, int ndkt, const LaunchIo& io, void* stream);
 // Turns raw histogram rows copied to buf ([nhist][stride], dtype as uploaded) into the
 // stored image in place: INT32 -> FP32, zero padding beyond nbins; writes seq to *flag
 // (host-mapped) if a count is not representable (|INT32| >= 2^24, non-finite float).

@@ -25,6 +25,12 @@
 // computed once per grid by one warp; the quarters' partial sums are added in a fixed order.
 // The arithmetic type is that of the path the table serves: FP64 for the plain path, FP32 for
 // the SPLIT path.
+//
+// What binds it: latency, then shared-memory loads (two CTAs on 152 SMs for one evaluation; each sum's
+// order is fixed, so the tables do not change with the layout).  The six arrays of a grid stand in shared
+// memory, the two derivative solves share their passes over f, a thread's four points share x_i, and the
+// three right-hand-side sums share G.  Measured (GB300, 684 points on the finer grid, FP32): 115 -> 65 us
+// a table against sums over arrays in global memory, one solve and one point per thread at a time.
 #include <cuda_runtime.h>
 
 #include "musr_dev.h"
@@ -36,10 +42,14 @@ constexpr int kB = 256;       // points per block of the solve
 constexpr int kQ = 4;         // threads per point
 constexpr int kT = kB * kQ;   // threads per CTA
 
+// Shared memory for a grid's six arrays: the finest FP32 grid.  With the static part (31 KB in FP64) and the
+// system's 1 KB it stays below the 227 KB of a CTA.
+constexpr int kDynSmem = 6 * 8200 * 4;
+
 template <class T>
 struct DktSmem {
   T tinv[kB];          // first column of the inverse of the block's Toeplitz matrix
-  T rhs[kB];
+  T rhs[2][kB];
   T part[kQ][3][kB];   // partial sums of the quarters of a point's threads
 };
 
@@ -53,42 +63,108 @@ __device__ __forceinline__ void quarter(int lo, int hi, int q, int* b, int* e) {
   *e = lo + ((q + 1) * n) / kQ;
 }
 
-// sum_{i=b}^{e-1} w[n - i] x[i] with four partial sums (independent FMA chains).
+// Sums sum_{i=b}^{e-1} w[n - i] x[i] run as four partial sums (independent FMA chains): i = b + 4 m + j into
+// the j-th, the last (e - b) % 4 into the first.
+
+// Three of them over one x, whose values are loaded once.
 template <class T>
-__device__ __forceinline__ T conv_range(const T* w, const T* x, int n, int b, int e) {
-  T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
+__device__ __forceinline__ void conv_range3(const T* u, const T* v, const T* w, const T* x, int n, int b, int e, T* ru,
+                                            T* rv, T* rw) {
+  T su[4], sv[4], sw[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) su[j] = sv[j] = sw[j] = T(0);
   int i = b;
-  for (; i + 3 < e; i += 4) {
-    s0 = fma(w[n - i], x[i], s0);
-    s1 = fma(w[n - i - 1], x[i + 1], s1);
-    s2 = fma(w[n - i - 2], x[i + 2], s2);
-    s3 = fma(w[n - i - 3], x[i + 3], s3);
+  for (; i + 3 < e; i += 4)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const T xi = x[i + j];
+      su[j] = fma(u[n - i - j], xi, su[j]);
+      sv[j] = fma(v[n - i - j], xi, sv[j]);
+      sw[j] = fma(w[n - i - j], xi, sw[j]);
+    }
+  for (; i < e; ++i) {
+    const T xi = x[i];
+    su[0] = fma(u[n - i], xi, su[0]);
+    sv[0] = fma(v[n - i], xi, sv[0]);
+    sw[0] = fma(w[n - i], xi, sw[0]);
   }
-  for (; i < e; ++i) s0 = fma(w[n - i], x[i], s0);
-  return (s0 + s1) + (s2 + s3);
+  *ru = (su[0] + su[1]) + (su[2] + su[3]);
+  *rv = (sv[0] + sv[1]) + (sv[2] + sv[3]);
+  *rw = (sw[0] + sw[1]) + (sw[2] + sw[3]);
 }
 
-// X[k], k = 1..K, holds the right-hand side R_k on entry and the solution of
-// a X_k - c sum_{i=1}^{k-1} f_{k-i} X_i = R_k on exit (X[0] is not read).
-template <class T>
-__device__ void solve_blocks(const T* f, T* X, int K, T c, DktSmem<T>& sm) {
-  const int r = threadIdx.x % kB, q = threadIdx.x / kB;
+// X_v[k], k = 1..K, v < NV, hold right-hand sides R_k on entry and the solutions of
+// a X_k - c sum_{i=1}^{k-1} f_{k-i} X_i = R_k on exit (X[0] is not read).  Two solves (NV = 2) share the
+// loads of f.  The history of the 256 points takes 256 threads: one (quarter, 64 residues) each and 4 points
+// 64 apart, whose quarter is the same range of i, so that x_i is loaded once for the four; each point's sum
+// is formed as above. 
+template <class T, int NV>
+__device__ void solve_blocks(const T* f, T* X0, T* X1, int K, T c, DktSmem<T>& sm) {
+  const int tid = threadIdx.x, r = tid % kB, q = tid / kB;
   for (int k0 = 1; k0 <= K; k0 += kB) {
-    const int k = k0 + r;
     int b, e;
-    quarter(1, k0, q, &b, &e);  // this thread's quarter of the history i = 1 .. k0 - 1
-    sm.part[q][0][r] = k <= K ? conv_range(f, X, k, b, e) : T(0);
+    if (tid < kB) {
+      const int hq = tid / 64, g = tid % 64;
+      quarter(1, k0, hq, &b, &e);  // this thread's quarter of the history i = 1 .. k0 - 1
+      T s[NV][4][4];
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) s[v][p][j] = T(0);
+      int last[4];  // the point itself, or the last one where the point lies beyond it
+#pragma unroll
+      for (int p = 0; p < 4; ++p) last[p] = min(k0 + g + 64 * p, K);
+      int i = b;
+      for (; i + 3 < e; i += 4)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const T x0 = X0[i + j], x1 = NV == 2 ? X1[i + j] : T(0);
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            const T w = f[last[p] - i - j];
+            s[0][p][j] = fma(w, x0, s[0][p][j]);
+            if (NV == 2) s[NV - 1][p][j] = fma(w, x1, s[NV - 1][p][j]);
+          }
+        }
+      for (; i < e; ++i) {
+        const T x0 = X0[i], x1 = NV == 2 ? X1[i] : T(0);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const T w = f[last[p] - i];
+          s[0][p][0] = fma(w, x0, s[0][p][0]);
+          if (NV == 2) s[NV - 1][p][0] = fma(w, x1, s[NV - 1][p][0]);
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+          sm.part[hq][v][g + 64 * p] =
+              k0 + g + 64 * p <= K ? (s[v][p][0] + s[v][p][1]) + (s[v][p][2] + s[v][p][3]) : T(0);
+    }
     __syncthreads();
-    if (q == 0)
-      sm.rhs[r] = k <= K ? X[k] + c * ((sm.part[0][0][r] + sm.part[1][0][r]) + (sm.part[2][0][r] + sm.part[3][0][r]))
-                         : T(0);
+    const int k = k0 + r;
+    if (q < NV) {
+      const T* X = q ? X1 : X0;
+      sm.rhs[q][r] = k <= K ? X[k] + c * ((sm.part[0][q][r] + sm.part[1][q][r]) + (sm.part[2][q][r] + sm.part[3][q][r]))
+                            : T(0);
+    }
     __syncthreads();
     quarter(0, r + 1, q, &b, &e);  // this thread's quarter of s = 0 .. r
-    T x = T(0);
-    for (int s = b; s < e; ++s) x = fma(sm.tinv[r - s], sm.rhs[s], x);
+    T x = T(0), y = T(0);
+#pragma unroll 4
+    for (int s = b; s < e; ++s) {
+      const T t = sm.tinv[r - s];
+      x = fma(t, sm.rhs[0][s], x);
+      if (NV == 2) y = fma(t, sm.rhs[1][s], y);
+    }
     sm.part[q][0][r] = x;
+    if (NV == 2) sm.part[q][1][r] = y;
     __syncthreads();
-    if (q == 0 && k <= K) X[k] = (sm.part[0][0][r] + sm.part[1][0][r]) + (sm.part[2][0][r] + sm.part[3][0][r]);
+    if (q < NV && k <= K)
+      (q ? X1 : X0)[k] = (sm.part[0][q][r] + sm.part[1][q][r]) + (sm.part[2][q][r] + sm.part[3][q][r]);
     __syncthreads();
   }
 }
@@ -120,6 +196,7 @@ __device__ void solve_grid(T D, T nu, T h, int K, T* f, T* fD, T* fN, T* G, T* G
       T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
       if (live) {
         int q = 0;
+#pragma unroll 4
         for (; q + 3 < r0; q += 4) {
           s0 = fma(f[rr - q], sm.tinv[q], s0);
           s1 = fma(f[rr - q - 1], sm.tinv[q + 1], s1);
@@ -129,10 +206,13 @@ __device__ void solve_grid(T D, T nu, T h, int K, T* f, T* fD, T* fN, T* G, T* G
         for (; q < r0; ++q) s0 = fma(f[rr - q], sm.tinv[q], s0);
       }
       T acc = (s0 + s1) + (s2 + s3), tr = T(0);
+      T fj = tid > 0 && tid <= K ? f[tid] : T(0);  // f[tid - j], loaded a step ahead of its use
       for (int j = 0; j < 32 && r0 + j < nr; ++j) {
+        const T next = tid > j + 1 && tid - j - 1 <= K ? f[tid - j - 1] : T(0);
         if (tid == j) tr = rr == 0 ? T(1) / a : ca * acc;
         const T tj = __shfl_sync(0xffffffffu, tr, j);
-        if (live && tid > j) acc = fma(f[tid - j], tj, acc);
+        if (live && tid > j) acc = fma(fj, tj, acc);
+        fj = next;
       }
       if (live) sm.tinv[rr] = tr;
       __syncwarp();
@@ -141,7 +221,7 @@ __device__ void solve_grid(T D, T nu, T h, int K, T* f, T* fD, T* fN, T* G, T* G
   // G: right-hand side b f_k (G_0 = 1 enters it through the trapezoid's end term)
   for (int k = tid; k <= K; k += kT) G[k] = k == 0 ? T(1) : b * f[k];
   __syncthreads();
-  solve_blocks(f, G, K, c, sm);
+  solve_blocks<T, 1>(f, G, static_cast<T*>(nullptr), K, c, sm);
   // right-hand sides of the derivatives, from the whole G:
   //   Delta: b fD_k + c sum fD_{k-i} G_i
   //   nu:    (h/2)(G_k + f_k) + b fN_k + h sum f_{k-i} G_i + c sum fN_{k-i} G_i
@@ -152,9 +232,7 @@ __device__ void solve_grid(T D, T nu, T h, int K, T* f, T* fD, T* fN, T* G, T* G
     quarter(1, k, q, &lo, &hi);
     T sD = T(0), sf = T(0), sN = T(0);
     if (k <= K) {
-      sD = conv_range(fD, G, k, lo, hi);
-      sf = conv_range(f, G, k, lo, hi);
-      sN = conv_range(fN, G, k, lo, hi);
+      conv_range3(fD, f, fN, G, k, lo, hi, &sD, &sf, &sN);
     }
     sm.part[q][0][r] = sD;
     sm.part[q][1][r] = sf;
@@ -172,8 +250,7 @@ __device__ void solve_grid(T D, T nu, T h, int K, T* f, T* fD, T* fN, T* G, T* G
     }
     __syncthreads();
   }
-  solve_blocks(f, GD, K, c, sm);
-  solve_blocks(f, GN, K, c, sm);
+  solve_blocks<T, 2>(f, GD, GN, K, c, sm);
 }
 
 // Counter increment with acquire-release semantics at GPU scope, and the matching fence
@@ -192,14 +269,16 @@ __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_re
 // thread's writes before thread 0's acquire-release increment; acquire: that increment and a
 // fence by every thread of the finishing CTA (no CTA waits for the other).
 template <class T>
-__global__ void __launch_bounds__(kT) dkt_table_kernel(const Job* __restrict__ jobs, int ndkt) {
+__global__ void __launch_bounds__(kT) dkt_table_kernel(const Job* __restrict__ jobs, int ndkt, LaunchIo io) {
   __shared__ DktSmem<T> sm;
   __shared__ int second;
+  extern __shared__ __align__(16) unsigned char dkt_dyn[];
   const int pair = blockIdx.x >> 1, part = blockIdx.x & 1;
   const Job& job = jobs[pair / ndkt];
   const int src = pair % ndkt;
   const HistSet& hs = *job.hs;
-  auto value = [&](int m) { return m >= 0 ? job.params[m] : hs.consts[-1 - m]; };
+  const double* params = io.params ? io.params + static_cast<int64_t>(pair / ndkt) * io.P : job.params;
+  auto value = [&](int m) { return m >= 0 ? params[m] : hs.consts[-1 - m]; };
   const double Dd = value(hs.dkt_src[src].x), nd = value(hs.dkt_src[src].y);
   const double rate = fmax(fmax(fabs(Dd), fabs(nd)), 0.05);
   const double span = hs.dkt_span > 0.0 ? hs.dkt_span : 1.0;
@@ -216,11 +295,24 @@ __global__ void __launch_bounds__(kT) dkt_table_kernel(const Job* __restrict__ j
   T* GD = G + (kDktMaxK + 1);
   T* GN = GD + (kDktMaxK + 1);
   const T D = static_cast<T>(Dd), nu = static_cast<T>(nd);
-  if (part == 0) {
-    solve_grid<T>(D, nu, static_cast<T>(0.5 * h), 2 * K, w, w + L, w + 2 * L, G2, GD2, GN2, sm);  // halved grid
+  // The grid's arrays live in shared memory where they fit (always in FP32, up to 4095 intervals in
+  // FP64), and only the solutions go to memory; else in the work space.
+  const int Kg = part == 0 ? 2 * K : K, Ls = Kg + 5;
+  T *gG = part == 0 ? G2 : G, *gD = part == 0 ? GD2 : GD, *gN = part == 0 ? GN2 : GN;
+  const T hg = static_cast<T>(part == 0 ? 0.5 * h : h);
+  if (6 * static_cast<size_t>(Ls) * sizeof(T) <= kDynSmem) {
+    T* a = reinterpret_cast<T*>(dkt_dyn);
+    solve_grid<T>(D, nu, hg, Kg, a, a + Ls, a + 2 * Ls, a + 3 * Ls, a + 4 * Ls, a + 5 * Ls, sm);
+    __syncthreads();
+    for (int k = threadIdx.x; k <= Kg; k += kT) {
+      gG[k] = a[3 * Ls + k];
+      gD[k] = a[4 * Ls + k];
+      gN[k] = a[5 * Ls + k];
+    }
   } else {
-    T* fc = w + 6 * L;
-    solve_grid<T>(D, nu, static_cast<T>(h), K, fc, fc + Lc, fc + 2 * Lc, G, GD, GN, sm);
+    T* fc = part == 0 ? w : w + 6 * L;
+    const int Lf = part == 0 ? L : Lc;
+    solve_grid<T>(D, nu, hg, Kg, fc, fc + Lf, fc + 2 * Lf, gG, gD, gN, sm);
   }
   __syncthreads();
   if (threadIdx.x == 0) second = (atom_add_acq_rel_u32(job.dkt_count + src, 1u) & 1u) != 0u;
@@ -242,13 +334,17 @@ __global__ void __launch_bounds__(kT) dkt_table_kernel(const Job* __restrict__ j
 
 }  // namespace
 
-int launch_dkt_tables(int precision, const Job* d_jobs, int njobs, int ndkt, void* stream) {
+int launch_dkt_tables(int precision, const Job* d_jobs, int njobs, int ndkt, const LaunchIo& io, void* stream) {
   if (ndkt <= 0 || njobs <= 0) return 0;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  auto launch = [&](auto kernel) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem) != cudaSuccess) return;
+    kernel<<<2 * njobs * ndkt, kT, kDynSmem, s>>>(d_jobs, ndkt, io);
+  };
   if (precision == 0)
-    dkt_table_kernel<double><<<2 * njobs * ndkt, kT, 0, s>>>(d_jobs, ndkt);
+    launch(dkt_table_kernel<double>);
   else
-    dkt_table_kernel<float><<<2 * njobs * ndkt, kT, 0, s>>>(d_jobs, ndkt);
+    launch(dkt_table_kernel<float>);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;  // the caller reads and clears the error
 }
 

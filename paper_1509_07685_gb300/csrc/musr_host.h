@@ -80,11 +80,8 @@ struct EvalBufs {
   Job first{};           // the first job of the table on the device (launches carry it)
   bool key_valid = false;
   int k_prec = -1, k_var = -1, k_mode = -1, k_grad = -1, k_nvec = -1;
-  const double* k_params = nullptr;
-  const double* k_dirs = nullptr;
   bool k_pieces = false;
   int k_grid = 0;  // the partition's grid (k_pieces)
-  double* k_out = nullptr;
 };
 
 // RAII: make `dev` current, restore the caller's device on exit.

@@ -38,6 +38,7 @@
 
 #include <cuda_runtime.h>
 
+#include <cstddef>
 #include <cstdint>
 #include <type_traits>
 
@@ -1863,13 +1864,22 @@ __device__ void enter_job(const LaunchHead& head, int ji, SM& sm) {
   __syncthreads();  // the job before is no longer read
   const int tid = threadIdx.x;
   const HistSet* src = ji == 0 ? head.first.hs : head.jobs[ji].hs;
-  if (ji == 0) {
-    if (tid < static_cast<int>(sizeof(Job) / 8))
-      reinterpret_cast<uint64_t*>(&sm.job)[tid] = reinterpret_cast<const uint64_t*>(&head.first)[tid];
-  } else {
-    static_assert(sizeof(Job) % 8 == 0 && sizeof(Job) / 8 <= kBlock, "a job in one step");
-    if (tid < static_cast<int>(sizeof(Job) / 8))
-      reinterpret_cast<uint64_t*>(&sm.job)[tid] = reinterpret_cast<const uint64_t*>(head.jobs + ji)[tid];
+  static_assert(sizeof(Job) % 8 == 0 && sizeof(Job) / 8 <= kBlock, "a job in one step");
+  if (tid < static_cast<int>(sizeof(Job) / 8)) {
+    const Job* j = ji == 0 ? &head.first : head.jobs + ji;
+    uint64_t w = reinterpret_cast<const uint64_t*>(j)[tid];
+    const LaunchIo& io = head.io;
+    if (tid == static_cast<int>(offsetof(Job, params) / 8)) {
+      if (head.nx > 0)
+        w = reinterpret_cast<uint64_t>(static_cast<const double*>(sm.x));
+      else if (io.params)
+        w = reinterpret_cast<uint64_t>(io.params + ji * io.P);
+    } else if (tid == static_cast<int>(offsetof(Job, out) / 8)) {
+      if (io.out) w = reinterpret_cast<uint64_t>(io.out + ji * (1 + io.P));
+    } else if (tid == static_cast<int>(offsetof(Job, dir) / 8)) {
+      if (io.dirs) w = reinterpret_cast<uint64_t>(io.dirs + ji * io.P);
+    }
+    reinterpret_cast<uint64_t*>(&sm.job)[tid] = w;
   }
   if (ji == 0 && head.nx > 0 && tid < head.nx) sm.x[tid] = head.x[tid];
   if (sm.hs_src != src) {
@@ -1879,10 +1889,6 @@ __device__ void enter_job(const LaunchHead& head, int ji, SM& sm) {
   }
   __syncthreads();
   if (tid == 0) sm.hs_src = src;  // read again only after another barrier
-  if (ji == 0 && head.nx > 0) {
-    if (tid == 0) sm.job.params = sm.x;
-    __syncthreads();
-  }
 }
 
 // The job of global item gi: by division where every job has per_job items, else the last job whose

@@ -360,7 +360,7 @@ extern "C" int musr_eval_noalloc(const void* d_counts, int dtype, int nhist, int
   e = cudaMemsetAsync(d_zero, 0, sizeof(unsigned) * (nchunks + 1), stream);
   if (e != cudaSuccess) return na_cuda(e, "cudaMemsetAsync(counters)");
   LaunchInfo info;
-  const LaunchHead head{&dT->job, 1, nitems, nitems, 0, job, {}};
+  const LaunchHead head{&dT->job, 1, nitems, nitems, 0, {}, job, {}};
   if (launch_eval(precision, hs.shape, mode, job.grad, head, num_sms, cuda_stream, &info))
     return na_cuda(cudaGetLastError(), "kernel launch");
   return MUSR_OK;

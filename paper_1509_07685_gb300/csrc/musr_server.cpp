@@ -534,7 +534,7 @@ int launch_lane(musr_server* s, int L) {
   for (const Launch& Lc : launches) {
     if (Lc.items == 0) continue;
     LaunchInfo info;
-    const LaunchHead head{d_jobs + Lc.first, Lc.njobs, Lc.items, 0, 0, lane.h_jobs[Lc.first], {}};
+    const LaunchHead head{d_jobs + Lc.first, Lc.njobs, Lc.items, 0, 0, {}, lane.h_jobs[Lc.first], {}};
     if (launch_eval(Lc.prec, Lc.shape, Lc.mode, 1, head, s->num_sms, s->stream, &info))
       return MUSR_ECUDA;
   }
