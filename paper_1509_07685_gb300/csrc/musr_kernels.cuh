@@ -805,23 +805,26 @@ __device__ void fp64_item(const Job& job, const HistSet& hs, int item, Smem& sm)
   // Warp (FP64 shuffles), then the CTA's warps in a fixed order (FP64).
   bad = __syncthreads_or(bad);
   const int w = tid >> 5, lane = tid & 31;
-  const double r0 = warp_sum_d(acc_v);
-  if (lane == 0) sm.dred[w][0] = r0;
   if (GRAD) {
-    const double r1 = warp_sum_d(acc_n0), r2 = warp_sum_d(acc_bkg);
-    if (lane == 0) {
-      sm.dred[w][1] = r1;
-      sm.dred[w][2] = r2;
-    }
+    double a[64];
+    a[0] = acc_v;
+    a[1] = acc_n0;
+    a[2] = acc_bkg;
 #pragma unroll
     for (int k = 0; k < kMaxTerms; ++k)
 #pragma unroll
       for (int m = 0; m < kMaxPrims; ++m)
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const double r = warp_sum_d(acc_p[k][m][q]);
-          if (lane == 0) sm.dred[w][3 + (k * kMaxPrims + m) * 2 + q] = r;
-        }
+        for (int q = 0; q < 2; ++q) a[3 + (k * kMaxPrims + m) * 2 + q] = acc_p[k][m][q];
+#pragma unroll
+    for (int i = 1 + kFp64Channels; i < 64; ++i) a[i] = 0.0;
+    warp_scatter_sum<64>(a);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (2 * lane + i < 1 + kFp64Channels) sm.dred[w][2 * lane + i] = a[i];
+  } else {
+    const double r0 = warp_sum_d(acc_v);
+    if (lane == 0) sm.dred[w][0] = r0;
   }
   __syncthreads();
   if (!dbg_ok(job.dbg, item >= 0 && item < job.nrows, kDbgPartial)) return;
@@ -1061,23 +1064,33 @@ __device__ void list_item(const Job& job, const HistSet& hs, int item, Smem& sm)
   // Warp (FP64 shuffles), then the CTA's warps in a fixed order (FP64): the FP64 path's rows.
   bad = __syncthreads_or(bad);
   const int w = tid >> 5, lane = tid & 31;
-  const double r0 = warp_sum_d(static_cast<double>(acc_v) - static_cast<double>(acc_c));
-  if (lane == 0) sm.dred[w][0] = r0;
+  const double v = widen(acc_v) - widen(acc_c);
   if (GRAD) {
-    const double r1 = warp_sum_d(acc_n0), r2 = warp_sum_d(acc_bkg);
-    if (lane == 0) {
-      sm.dred[w][1] = r1;
-      sm.dred[w][2] = r2;
+    constexpr int NC = 3 + 2 * LT * LP, NP = (NC + 31) / 32 * 32;
+    double a[NP];
+    a[0] = v;
+    a[1] = widen(acc_n0);
+    a[2] = widen(acc_bkg);
+#pragma unroll
+    for (int k = 0; k < LT; ++k)
+#pragma unroll
+      for (int m = 0; m < LP; ++m)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) a[3 + (k * LP + m) * 2 + q] = widen(acc_p[k][m][q]);
+#pragma unroll
+    for (int i = NC; i < NP; ++i) a[i] = 0.0;
+    warp_scatter_sum<NP>(a);
+    // the FP64 path's row layout; slots beyond LT x LP are 0
+    for (int c = lane; c < 1 + kFp64Channels; c += 32) sm.dred[w][c] = 0.0;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < NP / 32; ++i) {
+      const int c = lane * (NP / 32) + i, j = c - 3, km = j >> 1;
+      if (c < NC) sm.dred[w][c < 3 ? c : 3 + ((km / LP) * kMaxPrims + km % LP) * 2 + (j & 1)] = a[i];
     }
-#pragma unroll
-    for (int k = 0; k < kMaxTerms; ++k)
-#pragma unroll
-      for (int m = 0; m < kMaxPrims; ++m)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {  // the FP64 path's row layout; slots beyond LT x LP are 0
-          const double r = k < LT && m < LP ? warp_sum_d(acc_p[k < LT ? k : 0][m < LP ? m : 0][q]) : 0.0;
-          if (lane == 0) sm.dred[w][3 + (k * kMaxPrims + m) * 2 + q] = r;
-        }
+  } else {
+    const double r0 = warp_sum_d(v);
+    if (lane == 0) sm.dred[w][0] = r0;
   }
   __syncthreads();
   if (!dbg_ok(job.dbg, item >= 0 && item < job.nrows, kDbgPartial)) return;
