@@ -15,10 +15,10 @@
 //     to the others by one complex multiplication with the chunk's table of the factor over i
 //     steps (i < kRebase; a Gaussian's cross term exp(-S t i D) by one more, a running product);
 //   * 1/N and 1/max(d,1) are an approximate reciprocal and one third-order Newton step, the
-//     logarithm of d/N a table of 256 intervals and a fifth-degree series;
+//     logarithm of d/N a table of 1024 intervals and a fourth-degree series;
 //   * comparisons, selections and the widening of FP32 counts run on the integer pipe.
 // What is left per pair (M = 3, -2lnL with gradient): N 3, residual 1, 1/N 3, u 1, d/N 1,
-// logarithm 7, cost 2, G and W 4, V 3 = 25 instructions, and a ninth of the per-bin work.
+// logarithm 6, cost 2, G and W 4, V 3 = 24 instructions, and an eighth of the per-bin work.
 //
 // Measured (GB300, 8 x 65536 bins, -2lnL, two cosine terms): see eval64_kernel below.
 #pragma once
@@ -30,7 +30,7 @@ namespace kern {
 namespace {
 
 constexpr int kRebase = 32;      // bins of a thread between two fresh evaluations of the time factors
-constexpr int kLogTable = 256;   // intervals of the logarithm's table
+constexpr int kLogTable = 1024;  // intervals of the logarithm's table
 
 // One chunk's constants for the FP64 basis kernels.
 struct Chunk64 {
@@ -48,6 +48,7 @@ struct Chunk64 {
   // Kubo-Toyabe exponential, the envelope
   double2 q[kMaxTerms][kRebase];
   double qk[kMaxTerms][kRebase], qe[kRebase];
+  double td[kRebase];  // i steps of 256 bins as a time
   int safe;         // the products neither overflow nor start from an underflowed value
 };
 
@@ -88,21 +89,20 @@ __device__ __forceinline__ double recip(double x) {
 }
 
 // ln x by table and series (Tang's method, ACM TOMS 16 (1990) 378): x = 2^k m with m in
-// [0.70, 1.41); c of m's interval (1/256 of an octave's mantissa range) approximates 1/m, so
-// that ln x = k ln 2 - ln c + ln(1 + r), r = m c - 1, |r| < 2^-9, the last by its series to r^5
-// (remainder below 2^-56).  The table's first interval edge above 1 is 1 itself and -ln c
-// shrinks towards it, so the absolute error stays at 2^-53 |ln x| + 2^-56 there.  Arguments
+// [0.70, 1.41); c of m's interval (1/1024 of an octave's mantissa range) approximates 1/m, so
+// that ln x = k ln 2 - ln c + ln(1 + r), r = m c - 1, |r| < 2^-11, the last by its series to r^4
+// (remainder below 2^-57).  One interval begins at 1 and -ln c shrinks towards it, so the absolute
+// error stays at 2^-53 |ln x| + 2^-57 there.  Arguments
 // outside [2^-1000, 2^1000] (or not positive numbers) take CUDA's log.
 constexpr int kLogOff = 0x3fe6a000;  // high word of the table's lower end
 __device__ __forceinline__ double ln_tab(double x, const double2* tab) {
   const int hi = __double2hiint(x);
   if (static_cast<unsigned>(hi - 0x01700000) > 0x7d000000u) return log(x);
   const int tmp = hi - kLogOff, k = tmp >> 20;
-  const double2 t = tab[(tmp >> 12) & (kLogTable - 1)];
+  const double2 t = tab[(tmp >> 10) & (kLogTable - 1)];
   const double m = __hiloint2double(hi - (k << 20), __double2loint(x));
   const double r = __fma_rn(m, t.x, -1.0);
-  double q = __fma_rn(r, 0.2, -0.25);
-  q = __fma_rn(r, q, 1.0 / 3.0);
+  double q = __fma_rn(r, -0.25, 1.0 / 3.0);
   q = __fma_rn(r, q, -0.5);
   double l = __dadd_rn(__fma_rn(__dmul_rn(r, r), q, r), t.y);
   if (k != 0) l = __fma_rn(static_cast<double>(k), 0.69314718055994530942, l);
@@ -125,8 +125,8 @@ constexpr double neg_ln(double c) {
 constexpr LogTable make_log_table() {
   LogTable r{};
   for (int i = 0; i < kLogTable; ++i) {
-    // high words from 0x3fe6a000 in steps of 0x1000: mantissa 1 + w / 2^20, below 1 at half the scale
-    const int lo = kLogOff + (i << 12), up = lo + 0x1000;
+    // high words from 0x3fe6a000 in steps of 0x400: mantissa 1 + w / 2^20, below 1 at half the scale
+    const int lo = kLogOff + (i << 10), up = lo + 0x400;
     auto value = [](int hi) {
       const double m = 1.0 + (hi & 0xfffff) / 1048576.0;
       return (hi >> 20) == 0x3ff ? m : 0.5 * m;
@@ -259,6 +259,7 @@ __device__ void load_chunk64(const Job& job, const HistSet& hs, SM& sm) {
     }
   } else if (many && wp == 2 + kMaxTerms) {
     c.qe[i] = exp(-c.rate * (i * D));
+    c.td[i] = i * D;
   }
   if (tid < nh) {
     double g[kGamStride], gd[kGamStride];
@@ -432,6 +433,9 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
   const double dt = hs.dt_us;
   const bool f32 = hs.store == kStoreF32;
   const bool safe = c.safe != 0;
+  bool timed = false;  // some term's value needs the bin's time (Kubo-Toyabe factors)
+#pragma unroll
+  for (int k = 0; k < NT; ++k) timed = timed || (k < nterms && !Bs::tf(c.kinds, k) && c.kinds[k] != kTermPlain);
 
   double acc_v = 0.0;
   double gacc[G][NPH], sh[NT][4];
@@ -447,12 +451,17 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
 
   TimeFactors<SHAPE> tf;
   const int iters = min(hs.tile_bins / kBlock, (nhi - ts + kBlock - 1) / kBlock);
-  double nd = __dadd_rn(static_cast<double>(ts + tid), -cc.t0);  // bin - t0
+  double nd = 0.0, t_fresh = 0.0;  // bin - t0 and its time, of the last fresh bin
   for (int it = 0; it < iters; ++it) {
-    const int n = ts + it * kBlock + tid;
-    const double t = __dmul_rn(nd, dt);
+    const int n = ts + it * kBlock + tid, step = safe ? it & (kRebase - 1) : 0;
+    if (step == 0) {
+      nd = __dadd_rn(static_cast<double>(n), -cc.t0);
+      t_fresh = __dmul_rn(nd, dt);
+    }
+    double t = t_fresh;
+    if (step != 0 && (GRAD || timed)) t = __dadd_rn(t, c.td[step]);
     double E, Pc[NT], Ps[NT], dK[NT];
-    tf.at(job, hs, c, safe ? it & (kRebase - 1) : 0, iters > 1, nd, t, &E, Pc, Ps, dK);
+    tf.at(job, hs, c, step, iters > 1, nd, t, &E, Pc, Ps, dK);
     double Bf[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) Bf[m] = m == 0 ? E : 0.0;
@@ -570,7 +579,6 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
         if (c.S[k] != 0.0) sh[k][1] = fma(-h2, Dk, sh[k][1]);
       }
     }
-    nd = __dadd_rn(nd, static_cast<double>(kBlock));
   }
 
   // thread -> warp (scatter sum) -> CTA (FP64 tree) -> row
@@ -620,12 +628,13 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
 // decomposition is picked for that grid.
 // Measured on GB300 (a call with its copies, before: the term-list kernel with CUDA's library
 // functions per histogram and bin):
-//   8 x 65536 bins, two cosine terms, -2lnL value and gradient, one vector   467 ->   80 us
-//   1 x 16384 bins, one cosine term, -2lnL at 1000 vectors                  4116 -> 1114 us
+//   8 x 65536 bins, two cosine terms, -2lnL value and gradient, one vector   467 ->   79 us
+//   1 x 16384 bins, one cosine term, -2lnL at 1000 vectors                  4116 -> 1050 us
 //   8 x 65536 bins, Gauss-Newton products along 28 directions               8884 ->  849 us
 //   (the whole matrix: musr_gram64.cu)
-// The first of these executes 47 FP64 instructions per pair (16 of them fresh time factors, a CTA
-// having two iterations), the second 33, the third 31.
+// The first of these executes 46 FP64 instructions per pair (16 of them fresh time factors, a CTA
+// having two iterations), the second 30 (33, 1114 us, with a table of 256 intervals and the bin's time
+// formed in every bin), the third 31.
 template <int SHAPE, int MODE, bool GRAD>
 __global__ void __launch_bounds__(kBlock, 1) eval64_kernel(const __grid_constant__ LaunchHead head) {
   __shared__ Smem64 sm;
@@ -636,7 +645,8 @@ __global__ void __launch_bounds__(kBlock, 1) eval64_kernel(const __grid_constant
     sm.cc.chunk = -1;
     sm.hs_src = nullptr;
   }
-  if (MODE == 1) sm.logtab[threadIdx.x] = log_table.t[threadIdx.x];  // read after several barriers
+  if (MODE == 1)  // read after several barriers
+    for (int i = threadIdx.x; i < kLogTable; i += kBlock) sm.logtab[i] = log_table.t[i];
   const Job& job = sm.job;
   const HistSet& hs = sm.hs;
   int ji = -1;
