@@ -250,7 +250,12 @@ __device__ void solve_grid(T D, T nu, T h, int K, T* f, T* fD, T* fN, T* G, T* G
     }
     __syncthreads();
   }
-  solve_blocks<T, 2>(f, GD, GN, K, c, sm);
+  if constexpr (sizeof(T) == sizeof(float)) {
+    solve_blocks<T, 2>(f, GD, GN, K, c, sm);
+  } else {  // bound by the FP64 pipe, and 64 registers a thread do not hold two solves' sums
+    solve_blocks<T, 1>(f, GD, static_cast<T*>(nullptr), K, c, sm);
+    solve_blocks<T, 1>(f, GN, static_cast<T*>(nullptr), K, c, sm);
+  }
 }
 
 // Counter increment with acquire-release semantics at GPU scope, and the matching fence
