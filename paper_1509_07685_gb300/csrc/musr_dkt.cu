@@ -28,8 +28,8 @@
 //
 // What binds it: latency, then shared-memory loads (two CTAs on 152 SMs for one evaluation; each sum's
 // order is fixed, so the tables do not change with the layout).  The six arrays of a grid stand in shared
-// memory, the two derivative solves share their passes over f, a thread's four points share x_i, and the
-// three right-hand-side sums share G.  Measured (GB300, 684 points on the finer grid, FP32): 115 -> 65 us
+// memory, the two derivative solves share their passes over f (in FP32), a thread's four points share x_i,
+// and the three right-hand-side sums share G.  Measured (GB300, 684 points on the finer grid, FP32): 115 -> 65 us
 // a table against sums over arrays in global memory, one solve and one point per thread at a time.
 #include <cuda_runtime.h>
 
