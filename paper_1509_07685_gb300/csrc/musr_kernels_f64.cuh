@@ -31,6 +31,7 @@ namespace {
 
 constexpr int kRebase = 32;      // bins of a thread between two fresh evaluations of the time factors
 constexpr int kLogTable = 1024;  // intervals of the logarithm's table
+constexpr int kRatioHi = 0x3eb00000;  // high word of 2^-20
 
 // One chunk's constants for the FP64 basis kernels.
 struct Chunk64 {
@@ -542,9 +543,17 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
         } else {
           const double r = __dadd_rn(N, -d);
           if (positive(d)) {
-            if (!positive(N)) bad = 1;
             u = __dmul_rn(r, recip(N));
-            acc_v = __dadd_rn(acc_v, __fma_rn(d, ln_tab(__dadd_rn(1.0, -u), sm.logtab), r));
+            double x = __dadd_rn(1.0, -u);  // d/N
+            // Below 2^-20 the difference has lost d/N's digits (and below 2^-53 all of them): the
+            // quotient itself.  Above it the logarithm's error, 2^-53 N/d, times d stays at 2^-53 of
+            // the bin's N - d.
+            if (__double2hiint(x) < kRatioHi) {
+              x = __ddiv_rn(d, N);
+              u = __dadd_rn(1.0, -x);
+            }
+            if (!positive(N)) bad = 1;
+            acc_v = __dadd_rn(acc_v, __fma_rn(d, ln_tab(x, sm.logtab), r));
           } else {
             u = 1.0;
             acc_v = __dadd_rn(acc_v, r);

@@ -1,0 +1,53 @@
+"""The FP64 basis kernels where a cost is defined but its counts, model or rates lie far from 1, against
+the oracle: counts far below the model (fractional counts of FP64 histograms, growing rates) and far
+above it.  Tolerance: the FP64 path's, 1e-12 of the value and of each gradient scale; every term of the
+value is formed with a relative error of a few roundings of the larger of d and N."""
+import numpy as np
+import pytest
+
+import musr_inputs as mi
+import oracle
+from test_gpu_parity import _check_fp64
+
+pytestmark = pytest.mark.gpu
+
+# slots: 0 N0, 1 Nbkg, 2 A, 3 lambda, 4 nu, 5 phi, 6 sigma
+TERMS = {
+    "T1": [[("AMP", (2,)), ("EXP", (3,)), ("TFCOS", (4, 5))]],
+    "N1": [[("AMP", (2,)), ("EXP", (3,)), ("GAUSS", (6,))]],
+    "generic": [[("AMP", (2,)), ("EXP", (3,))], [("AMP", (2,)), ("GAUSS", (6,))]],
+}
+
+
+def _problem(terms, counts, truth, dt=0.02, fit=None):
+    nhist, nbins = counts.shape
+    rows = np.array([[0, 1, 2, 3, 4, 5, 6]] * nhist, np.int32)
+    return mi.Problem(counts, np.zeros(nhist), dt * 1000.0, fit or (0.0, nbins * dt), terms, rows, np.zeros(1), 7,
+                      np.array(truth), [f"p{i}" for i in range(7)])
+
+
+def _check(p, mode=1):
+    from paper_1509_07685_gb300 import binding as B
+    with B.Context(p) as ctx:
+        ref = oracle.cost(p, p.truth, mode)
+        assert np.isfinite(ref[0])
+        v, g, st = ctx.eval(p.truth, mode, B.MUSR_FP64)
+        assert st == B.MUSR_OK
+        _check_fp64(v, g, ref)
+        assert ctx.eval(p.truth, mode, B.MUSR_FP64, grad=False)[0] == v
+
+
+@pytest.mark.parametrize("shape", list(TERMS))
+def test_counts_far_below_the_model(musr_lib, shape):
+    rng = np.random.default_rng(5)
+    counts = 10.0 ** rng.uniform(-25.0, 1.0, size=(2, 611))
+    counts[:, ::7] = 0.0
+    _check(_problem(TERMS[shape], counts, [40.0, 1.5, 0.06, 0.4, 3.0, 17.0, 0.35]))
+
+
+@pytest.mark.parametrize("shape", ["N1", "generic"])
+@pytest.mark.parametrize("lam,n0", [(-3.3, 1.0), (-5.0, 40.0), (0.4, 1e18), (60.0, 1e-20)])
+def test_integer_counts_far_from_the_model(musr_lib, shape, lam, n0):
+    rng = np.random.default_rng(6)
+    counts = rng.poisson(3.0, size=(3, 611)).astype(np.float32)
+    _check(_problem(TERMS[shape], counts, [n0, 0.0, 0.3, lam, 3.0, 17.0, 0.1]))
