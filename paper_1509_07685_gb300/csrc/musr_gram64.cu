@@ -14,7 +14,8 @@
 // Measured on GB300 (8 x 65536 bins, 28 parameters, -2lnL, the whole call): 8.88 ms with the term-list
 // kernel's products, 0.85 ms with the basis kernel's, 0.137 ms here.
 // Up to 12 local slots (78 sums fill the registers); theories with more, and dynamic Kubo-Toyabe factors,
-// whose tables are solved for a job on the device, keep the products.
+// whose tables are solved for a job on the device, keep the products, as do theories with a primitive on
+// N0's slot.
 #include "musr_kernels_f64.cuh"
 
 namespace musr {
@@ -271,6 +272,10 @@ bool plan_of(const HistSet& hs, const bool* active, GramPlan* p) {
                   static_cast<unsigned char>(slot)};
   };
   auto fn = [](int k, int q) { return Bs::M + 6 * k + q; };
+  // The kernel forms N from slot 0's derivative (N = N0 J_0 + Nbkg), which is N / N0's only where nothing
+  // but N0 reads the slot; a theory whose primitives read it too keeps the products.
+  for (int i = hs.slot_ptr[0]; i < hs.slot_ptr[1]; ++i)
+    if (hs.contrib[hs.slot_list[i]].kind != kCN0) return false;
   for (int s = 0; s < hs.nslots && fits; ++s) {
     if (s != 0 && (!active[s] || hs.slot_ptr[s] == hs.slot_ptr[s + 1])) continue;
     if (nj == kGramSlots) return false;

@@ -1,0 +1,48 @@
+"""The FP64 Gauss-Newton matrix in one pass (musr_gram64.cu) for maps and theories beyond the plain ones,
+against the oracle's matrix and the products with unit vectors (1e-12 of sqrt(H_ii H_jj): the path's
+tolerance)."""
+import numpy as np
+import pytest
+
+import musr_inputs as mi
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _counts(nhist, nbins, seed=9):
+    rng = np.random.default_rng(seed)
+    return rng.poisson(30.0, size=(nhist, nbins)).astype(np.float64)
+
+
+def _check(p, modes=(0, 1)):
+    from paper_1509_07685_gb300 import binding as B
+    with B.Context(p) as ctx:
+        for mode in modes:
+            H, ref = ctx.gauss_newton(p.truth, mode, B.MUSR_FP64), oracle.gauss_newton(p, p.truth, mode)
+            _, prod, _ = ctx.gn_product(p.truth, np.eye(p.nparams), mode, B.MUSR_FP64)
+            d = np.sqrt(np.diag(ref))
+            tol = 1e-12 * np.outer(d, d) + 1e-300
+            assert np.all(np.abs(H - ref) <= tol), (mode, np.max(np.abs(H - ref) / tol))
+            assert np.all(np.abs(H - 0.5 * (prod + prod.T)) <= tol)
+
+
+@pytest.mark.parametrize("terms", [
+    [[("AMP", (0,)), ("EXP", (2,))]],                      # the amplitude reads N0's slot
+    [[("AMP", (2,)), ("EXP", (0,))]],                      # the rate does
+    [[("AMP", (2,)), ("TFCOS", (3, 0))]],                  # the phase
+    [[("AMP", (1,)), ("EXP", (2,))]],                      # the amplitude reads Nbkg's slot
+    [[("AMP", (2,)), ("GAUSS", (1,)), ("TFCOS", (3, 4))]],  # the width does
+])
+def test_primitives_on_the_first_slots(musr_lib, terms):
+    """N0 = 3, Nbkg = 0.4, A = 0.3 (N > 0 throughout)."""
+    truth = np.array([3.0, 0.4, 0.3, 1.7, 20.0])
+    rows = np.array([[0, 1, 2, 3, 4]] * 2, np.int32)
+    used = {0, 1} | {s for t in terms for _, slots in t for s in slots}
+    if 4 not in used:  # parameters nothing reads: constants
+        rows = np.where(np.isin(rows, list(used)), rows, -1 - rows)
+    idx = {s: i for i, s in enumerate(sorted(used))}
+    rows = np.array([[idx[v] if v >= 0 else v for v in r] for r in rows], np.int32)
+    p = mi.Problem(_counts(2, 700), np.zeros(2), 8.0, (0.0, 5.6), terms, rows, truth.copy(), len(idx),
+                   truth[sorted(used)], [f"p{i}" for i in idx])
+    _check(p)
