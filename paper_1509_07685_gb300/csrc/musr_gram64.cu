@@ -198,12 +198,11 @@ __global__ void __launch_bounds__(kBlock, 1) gram64_kernel(const __grid_constant
           const double N = fma(N0, J[0], Nbkg);
           double w;
           if (gp.mode == 2) {
-            w = cc.roww[hl] ? 2.0 * __ldg(static_cast<const double*>(cc.roww[hl]) + n)
-                            : (above_one(d) ? 2.0 * recip(d) : 2.0);
+            w = 2.0 * (cc.roww[hl] ? __ldg(static_cast<const double*>(cc.roww[hl]) + n) : count_weight(d));
           } else {
             if (!positive(d)) continue;
             if (!positive(N)) bad = 1;
-            const double y = recip(N);
+            const double y = recip_any(N);
             w = 2.0 * d * y * y;
           }
 #pragma unroll

@@ -74,19 +74,29 @@ struct Smem64 {
 // Arithmetic
 // ---------------------------------------------------------------------------------------------
 
-// Whether x > 0 and x > 1 (x not a NaN): doubles order like their bits for positive values.
+// Whether x > 0 (x not a NaN): doubles order like their bits for positive values.
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
-__device__ __forceinline__ bool above_one(double x) { return __double_as_longlong(x) > 0x3ff0000000000000LL; }
 
 // 1/x from PTX's approximate reciprocal y (relative error e0 about 2^-20) by the third-order
 // Newton (Householder) step y + y (e + e^2), e = 1 - x y: the error left is e0^3, below the
-// rounding of the last operation.  x neither 0 nor subnormal nor above 2^1022.
+// rounding of the last operation.  x neither 0 nor subnormal (rcp's result would be infinite) nor
+// above 2^1022 (it would be flushed to 0): recip_range(x).
+__device__ __forceinline__ bool recip_range(double x) {  // x in [2^-1022, 2^1022)
+  return static_cast<unsigned>(__double2hiint(x) - 0x00100000) < 0x7fc00000u;
+}
 __device__ __forceinline__ double recip(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   double e = __fma_rn(-x, y, 1.0);
   e = __fma_rn(e, e, e);
   return __fma_rn(y, e, y);
+}
+__device__ __forceinline__ double recip_any(double x) { return recip_range(x) ? recip(x) : __ddiv_rn(1.0, x); }
+// 1 / max(d, 1)
+__device__ __forceinline__ double count_weight(double d) {
+  const int hi = __double2hiint(d);
+  if (static_cast<unsigned>(hi - 0x3ff00000) < 0x3fe00000u) return recip(d);  // d in [1, 2^1022)
+  return hi < 0x7fd00000 ? 1.0 : __ddiv_rn(1.0, d);
 }
 
 // ln x by table and series (Tang's method, ACM TOMS 16 (1990) 378): x = 2^k m with m in
@@ -515,7 +525,7 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
         else
           d = __ldg(static_cast<const double*>(cc.rowp[hl]) + n);
         if (MODE == 0 || MODE == 2)
-          iv = cc.roww[hl] ? __ldg(static_cast<const double*>(cc.roww[hl]) + n) : (above_one(d) ? recip(d) : 1.0);
+          iv = cc.roww[hl] ? __ldg(static_cast<const double*>(cc.roww[hl]) + n) : count_weight(d);
         double N = gm[0];
 #pragma unroll
         for (int m = 0; m < M; ++m) N = __fma_rn(gm[1 + m], Bf[m], N);
@@ -530,7 +540,7 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
             cw = 0.0;
             if (positive(d)) {
               if (!positive(N)) bad = 1;
-              const double y = recip(N);
+              const double y = recip_any(N);
               cw = d * y * y;
             }
           }
@@ -547,12 +557,12 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
             double x = __dadd_rn(1.0, -u);  // d/N
             // Below 2^-20 the difference has lost d/N's digits (and below 2^-53 all of them): the
             // quotient itself.  Above it the logarithm's error, 2^-53 N/d, times d stays at 2^-53 of
-            // the bin's N - d.
-            if (__double2hiint(x) < kRatioHi) {
+            // the bin's N - d.  N outside recip's range comes here too.
+            if (__double2hiint(x) < kRatioHi || !recip_range(N)) {
               x = __ddiv_rn(d, N);
               u = __dadd_rn(1.0, -x);
+              if (!positive(N)) bad = 1;
             }
-            if (!positive(N)) bad = 1;
             acc_v = __dadd_rn(acc_v, __fma_rn(d, ln_tab(x, sm.logtab), r));
           } else {
             u = 1.0;

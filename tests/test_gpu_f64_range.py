@@ -51,3 +51,27 @@ def test_integer_counts_far_from_the_model(musr_lib, shape, lam, n0):
     rng = np.random.default_rng(6)
     counts = rng.poisson(3.0, size=(3, 611)).astype(np.float32)
     _check(_problem(TERMS[shape], counts, [n0, 0.0, 0.3, lam, 3.0, 17.0, 0.1]))
+
+
+def test_subnormal_model(musr_lib):
+    """N below 2^-1022 (no background, a tiny N0): finite with fractional counts."""
+    rng = np.random.default_rng(7)
+    counts = rng.uniform(0.5e-6, 2e-6, size=(2, 97))
+    _check(_problem(TERMS["N1"], counts, [1.3e-308, 0.0, 0.3, 0.4, 3.0, 17.0, 0.1]))
+
+
+@pytest.mark.parametrize("mode,count,bkg", [(1, 5.0, 6e307), (0, 6e307, 2.0)])
+def test_largest_counts_and_model(musr_lib, mode, count, bkg):
+    """One bin with N, or d, above 2^1022, where 1 / N and 1 / d are subnormal: -2lnL = 2 N and its gradient 2
+    along Nbkg; chi^2 = d and -2."""
+    from paper_1509_07685_gb300 import binding as B
+    p = _problem(TERMS["N1"], np.full((1, 4), count), [1.0, bkg, 0.3, 0.4, 3.0, 17.0, 0.1], fit=(0.019, 0.021))
+    with B.Context(p) as ctx:
+        assert ctx.bins_in_fit() == 1
+        v, g, st = ctx.eval(p.truth, mode, B.MUSR_FP64)
+        want, slope = (2.0 * bkg, 2.0) if mode else (count, -2.0)
+        assert st == B.MUSR_OK and abs(v / want - 1.0) <= 1e-12 and abs(g[1] - slope) <= 1e-12
+        assert ctx.eval(p.truth, mode, B.MUSR_FP64, grad=False)[0] == v
+        H, (_, prod, _) = ctx.gauss_newton(p.truth, mode, B.MUSR_FP64), ctx.gn_product(p.truth, np.eye(7), mode, B.MUSR_FP64)
+        curv = 2.0 * count / bkg / bkg if mode else 2.0 / count  # d^2 cost / dN^2
+        assert abs(H[1, 1] - curv) <= 1e-12 * curv + 1e-323 and abs(prod[1, 1] - curv) <= 1e-12 * curv + 1e-323
