@@ -221,6 +221,13 @@ __device__ void load_chunk64(const Job& job, const HistSet& hs, SM& sm) {
         S = fma(g, g, S);
         ds = fma(g, cc.ldir[0][ct.gauss_slot[i]], ds);
       }
+      // finite rates whose sum or square overflows: the largest double, so that 0 times it (time zero) is 0
+      constexpr double kBig = 1.7976931348623157e308;
+      bool finite = true;
+      for (int i = 0; i < ct.nexp; ++i) finite = finite && isfinite(cc.loc[0][ct.exp_slot[i]]);
+      for (int i = 0; i < ct.ngauss; ++i) finite = finite && isfinite(cc.loc[0][ct.gauss_slot[i]]);
+      if (finite && !isfinite(lam)) lam = lam > 0.0 ? kBig : -kBig;
+      if (finite && !isfinite(S)) S = kBig;
       if (Bs::MERGED && ct.amp_slot >= 0) bamp = cc.loc[0][ct.amp_slot];
       if (kind == kTermKT || kind == kTermLKT || kind == kTermDKT) {
         kt = cc.loc[0][ct.kt_slot];

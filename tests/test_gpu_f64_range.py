@@ -75,3 +75,13 @@ def test_largest_counts_and_model(musr_lib, mode, count, bkg):
         H, (_, prod, _) = ctx.gauss_newton(p.truth, mode, B.MUSR_FP64), ctx.gn_product(p.truth, np.eye(7), mode, B.MUSR_FP64)
         curv = 2.0 * count / bkg / bkg if mode else 2.0 / count  # d^2 cost / dN^2
         assert abs(H[1, 1] - curv) <= 1e-12 * curv + 1e-323 and abs(prod[1, 1] - curv) <= 1e-12 * curv + 1e-323
+
+
+@pytest.mark.parametrize("shape,lam,sigma", [("N1", 0.4, 1e170), ("generic", 0.4, 1e170), ("rates", 1.2e308, 0.1)])
+def test_rates_whose_combination_overflows(musr_lib, shape, lam, sigma):
+    """sigma^2 and a sum of rates beyond the double range: the factor is 1 at time zero and 0 after it."""
+    terms = [[("AMP", (2,)), ("EXP", (3,)), ("EXP", (3,))]] if shape == "rates" else TERMS[shape]
+    counts = np.random.default_rng(8).poisson(3.0, size=(2, 300)).astype(np.float64)
+    p = _problem(terms, counts, [4.0, 1.5, 0.3, lam, 3.0, 17.0, sigma])
+    for mode in (0, 1):
+        _check(p, mode)
