@@ -101,11 +101,14 @@ __device__ __forceinline__ double count_weight(double d) {
 
 // ln x by table and series (Tang's method, ACM TOMS 16 (1990) 378): x = 2^k m with m in
 // [0.70, 1.41); c of m's interval (1/1024 of an octave's mantissa range) approximates 1/m, so
-// that ln x = k ln 2 - ln c + ln(1 + r), r = m c - 1, |r| < 2^-11, the last by its series to r^4
-// (remainder below 2^-57).  One interval begins at 1 and -ln c shrinks towards it, so the absolute
-// error stays at 2^-53 |ln x| + 2^-57 there.  Arguments
+// that ln x = k ln 2 - ln c + ln(1 + r), r = m c - 1, |r| < h = 2^-11, the last by its series to r^4 with
+// r^5 / 5 folded into the cubic term as (3/20) h^2 r^3: what is left is below 2^-59 on [-h, h] and odd, so
+// that it does not add up over a sum of bins.  One interval holds 1 (h/2 below it, h above) with c = 1, so
+// that ln is exactly 0 there and the absolute error near it stays at 2^-53 |ln x| + 2^-57.  Measured on the host over 65536 Poisson bins of 1e5 / 1e6 / 1e7 counts: a -2lnL's relative error
+// 2.3e-14 / 4.7e-13 / 2.9e-12, those of log(d / N) itself; with c = 1 from 1 to 2^-10 above it, where r leaves
+// [-h, h], and the plain series 4.5e-13 / 1.1e-11 / 4.3e-11.  Arguments
 // outside [2^-1000, 2^1000] (or not positive numbers) take CUDA's log.
-constexpr int kLogOff = 0x3fe6a000;  // high word of the table's lower end
+constexpr int kLogOff = 0x3fe6a200;  // high word of the table's lower end
 __device__ __forceinline__ double ln_tab(double x, const double2* tab) {
   const int hi = __double2hiint(x);
   if (static_cast<unsigned>(hi - 0x01700000) > 0x7d000000u) return log(x);
@@ -113,7 +116,7 @@ __device__ __forceinline__ double ln_tab(double x, const double2* tab) {
   const double2 t = tab[(tmp >> 10) & (kLogTable - 1)];
   const double m = __hiloint2double(hi - (k << 20), __double2loint(x));
   const double r = __fma_rn(m, t.x, -1.0);
-  double q = __fma_rn(r, -0.25, 1.0 / 3.0);
+  double q = __fma_rn(r, -0.25, 1.0 / 3.0 + 3.0 / 20.0 / 4194304.0);
   q = __fma_rn(r, q, -0.5);
   double l = __dadd_rn(__fma_rn(__dmul_rn(r, r), q, r), t.y);
   if (k != 0) l = __fma_rn(static_cast<double>(k), 0.69314718055994530942, l);
@@ -122,7 +125,7 @@ __device__ __forceinline__ double ln_tab(double x, const double2* tab) {
 
 // The table, computed when the library is compiled (a logarithm per thread at every launch would
 // cost it 2 us): c = 1 / (midpoint of the interval) in 24 bits or fewer (1 for the interval that
-// begins at 1: ln is then exactly 0 at x = 1), and -ln c of that c by the series of atanh,
+// holds 1), and -ln c of that c by the series of atanh,
 // ln c = 2 (z + z^3/3 + ...), z = (c - 1)/(c + 1), |z| < 0.18, summed from its smallest term.
 struct LogTable {
   double2 t[kLogTable];
@@ -136,16 +139,17 @@ constexpr double neg_ln(double c) {
 constexpr LogTable make_log_table() {
   LogTable r{};
   for (int i = 0; i < kLogTable; ++i) {
-    // high words from 0x3fe6a000 in steps of 0x400: mantissa 1 + w / 2^20, below 1 at half the scale
+    // high words from kLogOff in steps of 0x400: mantissa 1 + w / 2^20, below 1 at half the scale
     const int lo = kLogOff + (i << 10), up = lo + 0x400;
     auto value = [](int hi) {
       const double m = 1.0 + (hi & 0xfffff) / 1048576.0;
       return (hi >> 20) == 0x3ff ? m : 0.5 * m;
     };
     const double mid = 0.5 * (value(lo) + value(up));
-    const double c = lo == 0x3ff00000 ? 1.0 : static_cast<double>(static_cast<float>(1.0 / mid));
+    const bool one = lo <= 0x3ff00000 && 0x3ff00000 < up;
+    const double c = one ? 1.0 : static_cast<double>(static_cast<float>(1.0 / mid));
     r.t[i].x = c;
-    r.t[i].y = lo == 0x3ff00000 ? 0.0 : neg_ln(c);
+    r.t[i].y = one ? 0.0 : neg_ln(c);
   }
   return r;
 }
