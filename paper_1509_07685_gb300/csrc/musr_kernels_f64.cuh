@@ -345,14 +345,17 @@ struct TimeFactors {
   using Bs = Basis<SHAPE>;
   static constexpr int NT = Bs::NT;
   // Per term at the last fresh bin: the factor a exp(-L t - S t^2/2) with its cosine and sine
-  // parts (fc, fs), a Gaussian's cross ratio of one step w (already in fc, fs for the steps made),
-  // and the same of a Kubo-Toyabe term's own exponential (fk, wk); the envelope (fE).
+  // parts (fc, fs), a Gaussian's cross ratio of one step 1 + w (already in fc, fs for the steps made),
+  // and the same of a Kubo-Toyabe term's own exponential (fk, wk); the envelope (fE).  The ratio is
+  // kept as its difference from 1: rounded to a double it would add its own error at every step, with
+  // one sign along a thread (root mean square of a factor over 32768 bins, sigma 0.05: 6.2e-16 against
+  // 1.5e-16; at sigma 0.3 7.1e-16 against 4.0e-16, 4.5e-16 for the factor evaluated in every bin).
   double fE, fc[NT], fs[NT], w[NT], fk[NT], wk[NT];
 
   __device__ __forceinline__ TimeFactors() {
     fE = 0.0;
 #pragma unroll
-    for (int k = 0; k < NT; ++k) fc[k] = fs[k] = fk[k] = 0.0, w[k] = wk[k] = 1.0;
+    for (int k = 0; k < NT; ++k) fc[k] = fs[k] = fk[k] = w[k] = wk[k] = 0.0;
   }
 
   __device__ __forceinline__ void at(const Job& job, const HistSet& hs, const Chunk64& c, int step, bool many, double nd,
@@ -365,7 +368,7 @@ struct TimeFactors {
         if (k >= nterms) continue;
         const double S = c.S[k];
         fc[k] = __dmul_rn(c.bamp[k], exp(-__dmul_rn(__fma_rn(__dmul_rn(0.5, S), t, c.lam[k]), t)));
-        if (S != 0.0 && many) w[k] = exp(-__dmul_rn(__dmul_rn(S, t), kBlock * hs.dt_us));
+        if (S != 0.0 && many) w[k] = expm1(-__dmul_rn(__dmul_rn(S, t), kBlock * hs.dt_us));
         if (Bs::tf(c.kinds, k)) {
           const double p = __dmul_rn(c.st_hi[k], nd);  // phase in turns, as a double-double
           const double pl = __fma_rn(c.st_lo[k], nd, __fma_rn(c.st_hi[k], nd, -p));
@@ -376,7 +379,7 @@ struct TimeFactors {
         } else if (c.kinds[k] == kTermKT) {
           const double z = __dmul_rn(c.kt[k], t);
           fk[k] = exp(-__dmul_rn(__dmul_rn(0.5, z), z));
-          if (many) wk[k] = exp(-__dmul_rn(__dmul_rn(__dmul_rn(c.kt[k], c.kt[k]), t), kBlock * hs.dt_us));
+          if (many) wk[k] = expm1(-__dmul_rn(__dmul_rn(__dmul_rn(c.kt[k], c.kt[k]), t), kBlock * hs.dt_us));
         } else if (c.kinds[k] == kTermLKT) {
           fk[k] = exp(-__dmul_rn(c.kt[k], t));
         }
@@ -392,14 +395,14 @@ struct TimeFactors {
       for (int k = 0; k < NT; ++k) {
         if (k >= nterms) continue;
         const double2 q = c.q[k][step];
-        if (c.S[k] != 0.0) fc[k] = __dmul_rn(fc[k], w[k]);
+        if (c.S[k] != 0.0) fc[k] = __fma_rn(fc[k], w[k], fc[k]);
         if (Bs::tf(c.kinds, k)) {
-          if (c.S[k] != 0.0) fs[k] = __dmul_rn(fs[k], w[k]);
+          if (c.S[k] != 0.0) fs[k] = __fma_rn(fs[k], w[k], fs[k]);
           xc[k] = __fma_rn(fc[k], q.x, -__dmul_rn(fs[k], q.y));
           xs[k] = __fma_rn(fc[k], q.y, __dmul_rn(fs[k], q.x));
         } else {
           xc[k] = __dmul_rn(fc[k], q.x);
-          if (c.kinds[k] == kTermKT) fk[k] = __dmul_rn(fk[k], wk[k]);
+          if (c.kinds[k] == kTermKT) fk[k] = __fma_rn(fk[k], wk[k], fk[k]);
           if (c.kinds[k] == kTermKT || c.kinds[k] == kTermLKT) kg[k] = __dmul_rn(fk[k], c.qk[k][step]);
         }
       }

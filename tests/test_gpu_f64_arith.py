@@ -86,3 +86,27 @@ def test_reciprocals(lib):
     bound = 2.0 ** -53 * (1 + 2.0 ** -6) * exact + np.longdouble(2.0) ** -1075
     assert np.all(np.abs(_map(lib, 2, x) - exact) <= bound)
     assert np.array_equal(_map(lib, 2, [0.0, -3.0, 0.25, 1.0]), np.ones(4))
+
+
+PLAIN, TF, KT = 1, 2, 3  # musr_dev.h
+
+
+@pytest.mark.parametrize("kind,sigma,kt", [(PLAIN, 0.05, 0.0), (TF, 0.05, 0.0), (KT, 0.0, 0.05)])
+def test_gaussian_factors_do_not_drift_from_a_fresh_bin(lib, kind, sigma, kt):
+    """The factor at a bin is the fresh bin's, times one rounding per step made since (31 at most, 15.5 on
+    average), times a table entry: with the handful of roundings of these two the root mean square over
+    all bins is that of a walk of 20 roundings, each uniform within 2^-53.  A step factor that is itself
+    rounded to a double would add its error once per step, all with one sign."""
+    iters, dt, nu = 128, 12.8 / 32768, 3.1
+    P = np.zeros((iters * 256, 2))
+    assert lib.f64_factors(kind, 0.0, sigma, kt, nu, dt, 0.0, iters, _ptr(P)) == 0
+    t = np.arange(iters * 256) * np.longdouble(dt)
+    if kind == KT:
+        u = (np.longdouble(kt) * t) ** 2
+        exact = (1 + 2 * (1 - u) * np.exp(-u / 2)) / 3
+        got = P[:, 0].astype(np.longdouble)
+    else:
+        exact = np.exp(-(np.longdouble(sigma) * t) ** 2 / 2)
+        got = np.hypot(P[:, 0].astype(np.longdouble), P[:, 1].astype(np.longdouble))
+    err = ((got - exact) / exact).astype(np.float64)
+    assert np.sqrt(np.mean(err ** 2)) <= np.sqrt(20.0 / 3.0) * 2.0 ** -53
