@@ -498,6 +498,7 @@ int compile(musr_ctx* ctx, int prec, int var) {
     p_cols.insert(p_cols.end(), pcols[p].begin(), pcols[p].end());
   }
   p_ptr[ctx->P] = static_cast<int>(p_cols.size());
+  hs.npcols = p_ptr[ctx->P];
   if (p_cols.empty()) p_cols.push_back(0);
   if (items.empty()) items.push_back(make_int2(0, 0));
   if (chunks.empty()) chunks.push_back(Chunk{});

@@ -200,6 +200,7 @@ struct alignas(16) HistSet {  // copied by 16-byte words into shared memory
   const int* col_chunk;    // [ncols] chunk of each column
   const int* p_ptr;        // [P + 1] CSR: columns contributing to parameter p
   const int* p_cols;
+  int npcols;              // entries of p_cols: p_ptr[P] (columns of constants and always-zero ones are in no list)
 };
 
 // A work piece of a launch-level partition (SPLIT basis kernels, batches): nit CTA iterations

@@ -1701,7 +1701,7 @@ __device__ void chunk_finalize(const Job& job, const HistSet& hs, SM& sm) {
   const int first_unused = unused_from<PREC, SHAPE>(cc.nh);
   int pp = 0, pc = 0;
   if (single && tid <= hs.P) pp = hs.p_ptr[tid];
-  if (single && tid < hs.ncols) pc = hs.p_cols[tid];
+  if (single && tid < hs.npcols && dbg_ok(job.dbg, tid < hs.p_ptr[hs.P], kDbgCol)) pc = hs.p_cols[tid];
   // the columns in use: the basis kernels' rows hold zeros for the histograms beyond the chunk's
   const int skip = first_unused < nout ? unused_columns<PREC, SHAPE>(cc.nh) : 0, ncol = nout - skip;
   if (tid < ncol * tpc) {

@@ -303,6 +303,7 @@ extern "C" int musr_eval_noalloc(const void* d_counts, int dtype, int nhist, int
       }
   T.p_ptr[0] = 0;
   for (int p = 0; p < nparams; ++p) T.p_ptr[p + 1] = T.p_ptr[p] + count[p];
+  hs.npcols = T.p_ptr[nparams];
   for (int p = 0; p < nparams; ++p) count[p] = T.p_ptr[p];
   for (int cc = 0; cc < col; ++cc) {
     const Chunk& ch = T.chunks[T.col_chunk[cc]];
