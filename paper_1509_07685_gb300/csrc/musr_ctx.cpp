@@ -1484,7 +1484,10 @@ static int gram_matrix(musr_ctx* ctx, const double* params, int mode, double* ou
   const size_t rows = static_cast<size_t>(musr::gram_rows(plan, hs.nchunks, ctx->num_sms)) * sizeof(double);
   if (ev.gram.bytes < rows && dalloc(ctx, ev.gram, rows)) return 1;  // beyond the budget: the products need less
   const bool in_launch = P <= musr::kHeadParams;
-  if (!in_launch && ev.params.bytes < P * sizeof(double)) return 1;  // its buffer comes with the first evaluation
+  if (!in_launch && ev.params.bytes < P * sizeof(double)) {
+    ev.key_valid = false;
+    if (dalloc(ctx, ev.params, P * sizeof(double))) return 1;
+  }
   if (ensure_uploaded(ctx, MUSR_FP64, var)) return 1;
   int rc;
   if ((rc = ensure_host(ctx, &ev.h_in, &ev.h_in_bytes, P * sizeof(double)))) return rc;

@@ -46,3 +46,21 @@ def test_primitives_on_the_first_slots(musr_lib, terms):
     p = mi.Problem(_counts(2, 700), np.zeros(2), 8.0, (0.0, 5.6), terms, rows, truth.copy(), len(idx),
                    truth[sorted(used)], [f"p{i}" for i in idx])
     _check(p)
+
+
+def test_more_parameters_than_a_launch_carries(musr_lib):
+    """Beyond 128 parameters they are copied to the device; the first call on a context takes the same
+    kernel as the next one (the same bits)."""
+    from paper_1509_07685_gb300 import binding as B
+    p = mi.cfg2(nhist=48, nbins=700, bin_width_ns=16.0, seed=4, n0=60.0)  # 4 + 3 x 48 parameters
+    assert p.nparams > 128
+    for mode in (0, 1):
+        with B.Context(p) as ctx:
+            H = ctx.gauss_newton(p.truth, mode, B.MUSR_FP64)
+            assert np.array_equal(ctx.gauss_newton(p.truth, mode, B.MUSR_FP64), H)
+            v, g, _ = ctx.eval(p.truth, mode, B.MUSR_FP64)  # the context's tables still hold
+            ref = oracle.cost(p, p.truth, mode)
+            assert abs(v - ref[0]) <= 1e-12 * abs(ref[0]) and np.all(np.abs(g - ref[1]) <= 1e-12 * ref[2] + 1e-300)
+        ref = oracle.gauss_newton(p, p.truth, mode)
+        d = np.sqrt(np.diag(ref))
+        assert np.all(np.abs(H - ref) <= 1e-12 * np.outer(d, d) + 1e-300)
