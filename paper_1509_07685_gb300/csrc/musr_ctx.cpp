@@ -121,6 +121,18 @@ size_t Arena::used() const {
   return used_;
 }
 
+// Gives back what only Gauss-Newton matrices hold: their rows, and the tables of the decomposition
+// that no evaluation has used.  A matrix waits for its kernels, so nothing of it is in flight.
+static void release_gram(musr_ctx* ctx) {
+  dfree(ctx, ctx->ev.gram);
+  if (ctx->ev.gram_var < 0) return;
+  Compiled& c = ctx->comp[MUSR_FP64][ctx->ev.gram_var];
+  ctx->ev.gram_var = -1;
+  dfree(ctx, c.tables);
+  c.d_hs = nullptr;
+  c.uploaded = false;
+}
+
 int dalloc(musr_ctx* ctx, DevBuf& b, size_t bytes) {
   dfree(ctx, b);
   if (bytes == 0) bytes = 16;
@@ -132,10 +144,17 @@ int dalloc(musr_ctx* ctx, DevBuf& b, size_t bytes) {
     ctx->used += bytes;
     return MUSR_OK;
   }
+  // what an earlier Gauss-Newton matrix holds is given back where another buffer needs the memory
+  if (ctx->budget && ctx->used + bytes > ctx->budget) release_gram(ctx);
   if (ctx->budget && ctx->used + bytes > ctx->budget)
     return fail(ctx, MUSR_ENOMEM, "device memory budget exceeded (" + std::to_string(ctx->used + bytes) +
                                       " > " + std::to_string(ctx->budget) + " bytes)");
   cudaError_t e = cudaMalloc(&b.p, bytes);
+  if (e != cudaSuccess && ctx->ev.gram.p) {
+    cudaGetLastError();
+    release_gram(ctx);
+    e = cudaMalloc(&b.p, bytes);
+  }
   if (e != cudaSuccess) {
     b.p = nullptr;
     cudaGetLastError();
@@ -293,6 +312,7 @@ std::vector<int64_t> grid_shifts(const musr_ctx* ctx) {
 }
 
 void free_compiled(musr_ctx* ctx, Compiled& c) {
+  if (ctx->ev.gram_var >= 0 && &c == &ctx->comp[MUSR_FP64][ctx->ev.gram_var]) ctx->ev.gram_var = -1;
   dfree(ctx, c.tables);
   std::vector<char>().swap(c.blob);
   c.d_hs = nullptr;
@@ -617,6 +637,7 @@ int pick_variant(musr_ctx* ctx, int prec, int nvec) {
 // key -- precision, decomposition, mode, grad, nvec -- changes; prepare_jobs)
 int ensure_eval(musr_ctx* ctx, int prec, int var, int nvec) {
   EvalBufs& ev = ctx->ev;
+  if (prec == MUSR_FP64 && var == ev.gram_var) ev.gram_var = -1;  // the evaluations' tables from here on
   int urc = ensure_uploaded(ctx, prec, var);
   if (urc) return urc;
   const HistSet& hs = ctx->comp[prec][var].hs;
@@ -1482,13 +1503,22 @@ static int gram_matrix(musr_ctx* ctx, const double* params, int mode, double* ou
   const int ne = musr::gram_values(plan.nj);
   const size_t nsum = static_cast<size_t>(hs.nchunks) * musr::kGroupMax * ne;
   const size_t rows = static_cast<size_t>(musr::gram_rows(plan, hs.nchunks, ctx->num_sms)) * sizeof(double);
-  if (ev.gram.bytes < rows && dalloc(ctx, ev.gram, rows)) return 1;  // beyond the budget: the products need less
   const bool in_launch = P <= musr::kHeadParams;
   if (!in_launch && ev.params.bytes < P * sizeof(double)) {
     ev.key_valid = false;
     if (dalloc(ctx, ev.params, P * sizeof(double))) return 1;
   }
+  const bool own_tables = !ctx->comp[MUSR_FP64][var].uploaded || ev.gram_var == var;
   if (ensure_uploaded(ctx, MUSR_FP64, var)) return 1;
+  if (own_tables) ev.gram_var = -1;  // not to be given back by the allocation below
+  // last, since another allocation may give it back; beyond the budget: the products, which need less
+  const bool fits = ev.gram.bytes >= rows || !dalloc(ctx, ev.gram, rows);
+  if (own_tables) ev.gram_var = var;
+  if (!fits) {
+    cudaStreamSynchronize(ctx->stream);  // the tables' copy
+    release_gram(ctx);
+    return 1;
+  }
   int rc;
   if ((rc = ensure_host(ctx, &ev.h_in, &ev.h_in_bytes, P * sizeof(double)))) return rc;
   if ((rc = ensure_host(ctx, &ev.h_out, &ev.h_out_bytes, nsum * sizeof(double)))) return rc;

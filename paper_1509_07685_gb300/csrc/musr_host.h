@@ -73,6 +73,7 @@ struct EvalBufs {
   DevBuf dkt, dkt_work;  // dynamic Kubo-Toyabe tables and their solve's scratch, per evaluation
   DevBuf dkt_count;      // their completion counters (zeroed once; each solve adds 2)
   DevBuf gram;           // rows of a Gauss-Newton matrix
+  int gram_var = -1;     // the FP64 decomposition whose tables only matrices have used, or -1
   DevBuf part;           // a launch-level partition: chunk rows, CTA offsets, pieces
   double* h_in = nullptr;
   double* h_out = nullptr;

@@ -64,3 +64,33 @@ def test_more_parameters_than_a_launch_carries(musr_lib):
         ref = oracle.gauss_newton(p, p.truth, mode)
         d = np.sqrt(np.diag(ref))
         assert np.all(np.abs(H - ref) <= 1e-12 * np.outer(d, d) + 1e-300)
+
+
+def test_matrix_scratch_is_given_back_within_a_budget(musr_lib):
+    """The smallest memory budget that holds the products of a matrix and then a batch holds the matrix and
+    then the batch too: the one-pass kernel's rows do not stay in the batch's way."""
+    from paper_1509_07685_gb300 import binding as B
+    p = mi.cfg2(nhist=8, nbins=6000, bin_width_ns=2.0, seed=5, n0=60.0)
+    X, eye = mi.jitter(p.truth, 1000, seed=5, lo=0.98, hi=1.02), np.eye(p.nparams)
+
+    def runs(budget, matrix):
+        try:
+            with B.Context(p, hbm_budget_bytes=budget) as ctx:
+                matrix(ctx)
+                return ctx.eval_batch(X, 1, B.MUSR_FP64)
+        except B.MusrError as e:
+            assert e.status == B.MUSR_ENOMEM
+            return None
+
+    products = lambda ctx: ctx.gn_product(p.truth, eye, 1, B.MUSR_FP64)
+    lo, hi = 1 << 16, 1 << 28
+    assert runs(hi, products)
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if runs(mid, products) else (mid, hi)
+    got = runs(hi, lambda ctx: ctx.gauss_newton(p.truth, 1, B.MUSR_FP64))
+    assert got
+    for i in (0, 999):
+        ref = oracle.cost(p, X[i], 1)
+        assert abs(got[0][i] - ref[0]) <= 1e-12 * abs(ref[0])
+        assert np.all(np.abs(got[1][i] - ref[1]) <= 1e-12 * ref[2] + 1e-300)
