@@ -218,7 +218,10 @@ int musr_eval_batch(musr_ctx* ctx, const double* params, int nvec, int nparams, 
  * tensors): d_params is device [nvec][nparams] FP64, d_out device
  * [nvec][1 + nparams] FP64 (value, then gradient; with_grad == 0 writes the
  * value only).  Asynchronous: enqueued on the context's stream, nothing is
- * copied or synchronised.  A +inf value marks an undefined likelihood. */
+ * copied or synchronised.  A +inf value marks an undefined likelihood.  On a
+ * stream that is capturing, a call that another evaluation has prepared (same nvec,
+ * mode, precision, with_grad as the context's last one) is recorded; others need
+ * set-up and return MUSR_ESTATE. */
 int musr_eval_device(musr_ctx* ctx, const double* d_params, int nvec, int mode, int precision,
                      int with_grad, double* d_out);
 

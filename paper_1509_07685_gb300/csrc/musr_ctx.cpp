@@ -852,6 +852,17 @@ struct LaunchPlan {
   const double* x = nullptr;  // one evaluation's parameters (host), to go with the launch
 };
 
+// A capturing stream would record the set-up of a launch (the tables' copy, cleared counters) instead of
+// doing it, and the next launch outside the graph would run on memory that was never written.
+int refuse_capture(musr_ctx* ctx) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(ctx->stream, &cap);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaStreamIsCapturing");
+  if (cap == cudaStreamCaptureStatusNone) return MUSR_OK;
+  return fail(ctx, MUSR_ESTATE, "the context's stream is capturing and the call needs set-up (tables, buffers): make "
+                                "the same call once before the capture");
+}
+
 int plan_launch(musr_ctx* ctx, int prec, int mode, int grad, int nvec, const double* d_params, double* d_out,
                 const double* d_dirs, LaunchPlan* L) {
   if (ctx->asym && prec == MUSR_SPLIT && mode == MUSR_CHI2) mode = 4;  // SPLIT kernels: weighted chi^2
@@ -873,6 +884,7 @@ int plan_launch(musr_ctx* ctx, int prec, int mode, int grad, int nvec, const dou
     L->grid = ev.k_grid;
     return MUSR_OK;
   }
+  if (const int rc = refuse_capture(ctx)) return rc;
   // Batches of plain evaluations on the SPLIT basis kernels may take a launch-level partition.
   Partition part;
   L->pieces = prec == MUSR_SPLIT && nvec >= 2 && (mode == 0 || mode == 1 || mode == 4) &&
@@ -1499,6 +1511,7 @@ static int gram_matrix(musr_ctx* ctx, const double* params, int mode, double* ou
     for (int s = 0; s < ctx->nslots; ++s) active[s] |= ctx->map[static_cast<size_t>(h) * ctx->nslots + s] >= 0;
   musr::GramPlan plan;
   if (!musr::gram_plan(hs, active, mode + 2, &plan)) return 1;
+  if (const int rc = refuse_capture(ctx)) return rc;
   EvalBufs& ev = ctx->ev;
   const int ne = musr::gram_values(plan.nj);
   const size_t nsum = static_cast<size_t>(hs.nchunks) * musr::kGroupMax * ne;
