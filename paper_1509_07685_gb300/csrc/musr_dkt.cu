@@ -97,13 +97,43 @@ __device__ __forceinline__ void conv_range3(const T* u, const T* v, const T* w, 
 // a X_k - c sum_{i=1}^{k-1} f_{k-i} X_i = R_k on exit (X[0] is not read).  Two solves (NV = 2) share the
 // loads of f.  The history of the 256 points takes 256 threads: one (quarter, 64 residues) each and 4 points
 // 64 apart, whose quarter is the same range of i, so that x_i is loaded once for the four; each point's sum
-// is formed as above. 
+// is formed as above.  A last block with few points takes a thread per (quarter, point) instead, and no
+// thread for the points beyond it: four points to a thread cost the same for 32 points as for 256.  FP64 is
+// bound by its multiply-adds, so every partial block goes this way (an FP64 call whose grids have 400 and 800
+// intervals 847 -> 732 us, 798 us with a point per thread throughout); FP32 by its loads, 5 for 4
+// multiply-adds with four points to a thread and 2 for each with one: from 160 points on four are the better.
 template <class T, int NV>
 __device__ void solve_blocks(const T* f, T* X0, T* X1, int K, T c, DktSmem<T>& sm) {
   const int tid = threadIdx.x, r = tid % kB, q = tid / kB;
   for (int k0 = 1; k0 <= K; k0 += kB) {
     int b, e;
-    if (tid < kB) {
+    const int live = K + 1 - k0;
+    if (live <= (sizeof(T) == sizeof(float) ? 160 : kB - 1)) {
+      quarter(1, k0, q, &b, &e);
+      if (r < live) {
+        T s[NV][4];
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) s[v][j] = T(0);
+        const T* w = f + k0 + r;
+        int i = b;
+        for (; i + 3 < e; i += 4)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const T wi = w[-i - j];
+            s[0][j] = fma(wi, X0[i + j], s[0][j]);
+            if (NV == 2) s[NV - 1][j] = fma(wi, X1[i + j], s[NV - 1][j]);
+          }
+        for (; i < e; ++i) {
+          const T wi = w[-i];
+          s[0][0] = fma(wi, X0[i], s[0][0]);
+          if (NV == 2) s[NV - 1][0] = fma(wi, X1[i], s[NV - 1][0]);
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) sm.part[q][v][r] = (s[v][0] + s[v][1]) + (s[v][2] + s[v][3]);
+      }
+    } else if (tid < kB) {
       const int hq = tid / 64, g = tid % 64;
       quarter(1, k0, hq, &b, &e);  // this thread's quarter of the history i = 1 .. k0 - 1
       T s[NV][4][4];
