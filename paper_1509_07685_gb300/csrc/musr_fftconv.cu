@@ -410,8 +410,14 @@ bool plan_axis(FftAxis* ax, int m) {
   return true;
 }
 
-// Columns per block: 64 KB of shared memory at most where that leaves one (three blocks per SM).
-int columns_of(int mp) { return mp <= 256 ? 8 : mp <= 512 ? 4 : mp <= 1024 ? 2 : 1; }
+// Columns per block: 64 KB of shared memory at most where that leaves one (three blocks per SM), fewer where
+// `sets` sets of n columns would leave SMs without a block.
+// Measured: a solve of 1 x 1 x 300 91 -> 52 us, 73 with the library's transforms.
+int columns_of(int mp, int64_t n, int64_t sets, int num_sms) {
+  int c = mp <= 256 ? 8 : mp <= 512 ? 4 : mp <= 1024 ? 2 : 1;
+  while (c > 1 && (n + c - 1) / c * sets < num_sms) c /= 2;
+  return c;
+}
 
 template <class K>
 cudaError_t allow_smem(K kernel, size_t bytes) {
@@ -453,9 +459,9 @@ cudaError_t run_x(const FftConv* c, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-#define MUSR_BY_COLUMNS(mp, f, ...)       \
+#define MUSR_BY_COLUMNS(columns, f, ...)  \
   [&] {                                   \
-    switch (columns_of(mp)) {             \
+    switch (columns) {                    \
       case 8:                             \
         return f<8>(__VA_ARGS__);         \
       case 4:                             \
@@ -469,10 +475,18 @@ cudaError_t run_x(const FftConv* c, cudaStream_t s) {
 
 }  // namespace
 
-bool fftconv_plan(FftConv* c, int mx, int my, int mz) {
+bool fftconv_plan(FftConv* c, int mx, int my, int mz, int num_sms) {
+  c->num_sms = num_sms;
   // grid limits: the y kernels' planes are a grid's second dimension
   if (mx > 65535 || !plan_axis(&c->x, mx) || !plan_axis(&c->y, my) || !plan_axis(&c->z, mz)) return false;
   c->nzc = c->z.mp + 1;
+  // A block holds a line of a long axis by itself and takes 26 (y, z) or 55 (x) FP64 instructions per point of
+  // it, 60 us at 2048 points and 250 us at 4096 over a solve's kernels, however few the lines; the library splits
+  // a line.  Measured, one solve with its wait, ours and the library's: 2048 x 4 x 4 159 / 136 us, 2048 x 8 x 8
+  // 215 / 250, 4096 x 2 x 2 267 / 107, 4096 x 4 x 4 283 / 203, 4096 x 8 x 8 395 / 470, 1500 x 1 x 1 116 / 155.
+  const int longest = c->x.mp > c->y.mp ? (c->x.mp > c->z.mp ? c->x.mp : c->z.mp) : (c->y.mp > c->z.mp ? c->y.mp : c->z.mp);
+  const int64_t lines = static_cast<int64_t>(c->x.mp) * c->y.mp * c->z.mp / longest;
+  if (longest > 1536 && lines < 32) return false;
   return 8.0 * c->x.mp * c->y.mp * c->z.mp < 4294967296.0;
 }
 
@@ -539,11 +553,14 @@ cudaError_t fftconv_set_kernel(FftConv* c, const double2* hat, double scale, cud
 }
 
 cudaError_t fftconv_solve(const FftConv* c, const double* rho, double* phi, cudaStream_t s) {
-  cudaError_t e = MUSR_BY_COLUMNS(c->z.mp, run_z, c, rho, phi, true, s);
-  if (e == cudaSuccess) e = MUSR_BY_COLUMNS(c->y.mp, run_y, c, true, s);
-  if (e == cudaSuccess) e = MUSR_BY_COLUMNS(c->x.mp, run_x, c, s);
-  if (e == cudaSuccess) e = MUSR_BY_COLUMNS(c->y.mp, run_y, c, false, s);
-  if (e == cudaSuccess) e = MUSR_BY_COLUMNS(c->z.mp, run_z, c, rho, phi, false, s);
+  const int64_t rows = static_cast<int64_t>(c->x.m) * c->y.m;
+  const int cz = columns_of(c->z.mp, (rows + 1) / 2, 1, c->num_sms), cy = columns_of(c->y.mp, c->nzc, c->x.m, c->num_sms);
+  const int cx = columns_of(c->x.mp, 2LL * c->y.mp * c->nzc, 1, c->num_sms);
+  cudaError_t e = MUSR_BY_COLUMNS(cz, run_z, c, rho, phi, true, s);
+  if (e == cudaSuccess) e = MUSR_BY_COLUMNS(cy, run_y, c, true, s);
+  if (e == cudaSuccess) e = MUSR_BY_COLUMNS(cx, run_x, c, s);
+  if (e == cudaSuccess) e = MUSR_BY_COLUMNS(cy, run_y, c, false, s);
+  if (e == cudaSuccess) e = MUSR_BY_COLUMNS(cz, run_z, c, rho, phi, false, s);
   return e;
 }
 

@@ -23,6 +23,7 @@ struct FftAxis {
 
 struct FftConv {
   FftAxis x, y, z;
+  int num_sms = 1;
   int nzc = 0;              // spectrum columns per (x, y) line: mp_z + 1
   double2* a = nullptr;     // [m_x][m_y][nzc]
   double2* b = nullptr;     // [m_x][2 mp_y][nzc]
@@ -30,8 +31,8 @@ struct FftConv {
   void* tables = nullptr;   // twiddles and positions
 };
 
-// Axis lengths for a mesh; false where an axis is too long for these kernels.
-bool fftconv_plan(FftConv* c, int mx, int my, int mz);
+// Axis lengths for a mesh; false where an axis is too long for these kernels, or long with few lines.
+bool fftconv_plan(FftConv* c, int mx, int my, int mz, int num_sms);
 // The tables on the device; the buffers of a solve.
 cudaError_t fftconv_tables(FftConv* c);
 cudaError_t fftconv_buffers(FftConv* c);

@@ -351,7 +351,7 @@ int musr_poisson_create(musr_poisson** out, int device, int mx, int my, int mz, 
   cudaError_t e = cudaMalloc(&ps->rho, sizeof(double) * nm);
   if (e == cudaSuccess) e = cudaMalloc(&ps->phi, sizeof(double) * nm);
   if (e != cudaSuccess) return fail_create(cuda_err(ps, e, "cudaMalloc"));
-  if (precision == MUSR_FP64 && musr::fftconv_plan(&ps->conv, mx, my, mz)) {
+  if (precision == MUSR_FP64 && musr::fftconv_plan(&ps->conv, mx, my, mz, ps->num_sms)) {
     ps->pruned = true;
     const int rc = setup_pruned(ps);
     if (rc) return fail_create(rc);
