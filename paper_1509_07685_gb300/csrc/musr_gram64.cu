@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kBlock, 1) gram64_kernel(const __grid_constant
           const double N = fma(N0, J[0], Nbkg);
           double w;
           if (gp.mode == 2) {
-            w = 2.0 * (cc.roww[hl] ? __ldg(static_cast<const double*>(cc.roww[hl]) + n) : count_weight(d));
+            w = 2.0 * (cc.roww[hl] ? __ldg(static_cast<const double*>(cc.roww[hl]) + n) : count_weight(d, f32));
           } else {
             if (!positive(d)) continue;
             if (!positive(N)) bad = 1;

@@ -74,8 +74,9 @@ struct Smem64 {
 // Arithmetic
 // ---------------------------------------------------------------------------------------------
 
-// Whether x > 0 (x not a NaN): doubles order like their bits for positive values.
+// Whether x > 0 and x > 1 (x not a NaN): doubles order like their bits for positive values.
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool above_one(double x) { return __double_as_longlong(x) > 0x3ff0000000000000LL; }
 
 // 1/x from PTX's approximate reciprocal y (relative error e0 about 2^-20) by the third-order
 // Newton (Householder) step y + y (e + e^2), e = 1 - x y: the error left is e0^3, below the
@@ -91,12 +92,14 @@ __device__ __forceinline__ double recip(double x) {
   e = __fma_rn(e, e, e);
   return __fma_rn(y, e, y);
 }
-__device__ __forceinline__ double recip_any(double x) { return recip_range(x) ? recip(x) : __ddiv_rn(1.0, x); }
-// 1 / max(d, 1)
-__device__ __forceinline__ double count_weight(double d) {
-  const int hi = __double2hiint(d);
-  if (static_cast<unsigned>(hi - 0x3ff00000) < 0x3fe00000u) return recip(d);  // d in [1, 2^1022)
-  return hi < 0x7fd00000 ? 1.0 : __ddiv_rn(1.0, d);
+// The division of values outside that range.  A call: inlined, its instructions are predicated into the
+// loop over bins, and one that is predicated off takes the FP64 pipe all the same.
+__device__ __noinline__ double divide(double a, double b) { return __ddiv_rn(a, b); }
+__device__ __forceinline__ double recip_any(double x) { return recip_range(x) ? recip(x) : divide(1.0, x); }
+// 1 / max(d, 1); only FP64 stores (f32 false) can hold counts above recip's range.
+__device__ __forceinline__ double count_weight(double d, bool f32) {
+  if (!f32 && __double2hiint(d) >= 0x7fd00000) return divide(1.0, d);
+  return above_one(d) ? recip(d) : 1.0;
 }
 
 // ln x by table and series (Tang's method, ACM TOMS 16 (1990) 378): x = 2^k m with m in
@@ -539,7 +542,7 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
         else
           d = __ldg(static_cast<const double*>(cc.rowp[hl]) + n);
         if (MODE == 0 || MODE == 2)
-          iv = cc.roww[hl] ? __ldg(static_cast<const double*>(cc.roww[hl]) + n) : count_weight(d);
+          iv = cc.roww[hl] ? __ldg(static_cast<const double*>(cc.roww[hl]) + n) : count_weight(d, f32);
         double N = gm[0];
 #pragma unroll
         for (int m = 0; m < M; ++m) N = __fma_rn(gm[1 + m], Bf[m], N);
@@ -573,7 +576,7 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
             // quotient itself.  Above it the logarithm's error, 2^-53 N/d, times d stays at 2^-53 of
             // the bin's N - d.  N outside recip's range comes here too.
             if (__double2hiint(x) < kRatioHi || !recip_range(N)) {
-              x = __ddiv_rn(d, N);
+              x = divide(d, N);
               u = __dadd_rn(1.0, -x);
               if (!positive(N)) bad = 1;
             }

@@ -11,7 +11,7 @@ __global__ void elementwise(int what, const double* __restrict__ x, double* __re
   for (int i = threadIdx.x; i < kLogTable; i += blockDim.x) tab[i] = log_table.t[i];
   __syncthreads();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    y[i] = what == 0 ? ln_tab(x[i], tab) : what == 1 ? recip_any(x[i]) : count_weight(x[i]);
+    y[i] = what == 0 ? ln_tab(x[i], tab) : what == 1 ? recip_any(x[i]) : count_weight(x[i], false);
 }
 
 // One CTA through `iters` iterations of kBlock bins of a one-term theory without an envelope: P of
