@@ -137,7 +137,7 @@ struct Contrib {
 // Only chunks with at least one bin in the fit range are listed.
 struct Chunk {
   int first;      // index into HistSet::hist_index of its first histogram
-  int nh;         // number of histograms (<= kGroupMax, 1 on the FP64 path)
+  int nh;         // number of histograms (<= kGroupMax; 1 where the theory has no basis form)
   int nlo, nhi;   // bins [nlo, nhi) in the fit (shared by the chunk)
   int item0;      // first work item of the chunk (HistSet-local)
   int ntiles;
@@ -194,7 +194,7 @@ struct alignas(16) HistSet {  // copied by 16-byte words into shared memory
   int nitems;
   int tile_bins;           // bins per tile
   int group;               // histograms per chunk at most
-  int nch;                 // reduction channels per item (SPLIT: per shape; FP64: 2 + 32)
+  int nch;                 // reduction channels per item (basis forms: per shape; term lists: 2 + 32)
   int pstride;             // doubles per partial row: 1 + nch
   int ncols;               // slot columns: sum over chunks of nh * nslots
   const int* col_chunk;    // [ncols] chunk of each column
@@ -275,7 +275,6 @@ struct LaunchHead {
   double x[kHeadParams];
 };
 
-// Launchers (host side of musr_kernels.cu).  All enqueue on `stream`.
 // The Gauss-Newton matrix of a basis theory in one pass (musr_gram64.cu): the local slots j < nj
 // (slot 0, N0, first) and the derivative of N by each as a sum over entries [ptr[j], ptr[j + 1]) of a
 // coefficient per histogram times a function of time.
@@ -305,6 +304,7 @@ int64_t gram_rows(const GramPlan& plan, int nchunks, int num_sms);
 int launch_gram(int shape, const GramPlan& plan, const LaunchHead& head, int nchunks, double* rows, double* sums,
                 int num_sms, void* stream);
 
+// Launchers (host side of musr_kernels.cu).  All enqueue on `stream`.
 struct LaunchInfo {
   int grid;
   int block;

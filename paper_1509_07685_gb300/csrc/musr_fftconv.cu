@@ -28,7 +28,7 @@
 // The half length mp is the product of 2, 3, 5 and 7 at or above m that needs the fewest
 // instructions (m itself where it is such a product): the padded circular length 2 mp >= 2 m gives
 // the same linear convolution.  Axes whose half length would exceed 4096 stay with the library's
-// transform (a block could not hold a line's two halves).
+// transform (a block could not hold a line's two halves), as do long axes with few lines (fftconv_plan).
 #include "musr_fftconv.h"
 
 #include <cmath>

@@ -624,7 +624,7 @@ __device__ void load_tile_at(int ts, const HistSet& hs, int prec, SM& sm) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// FP64 path: one histogram per chunk, every operation in FP64, term list as given.
+// FP64 term list: one histogram per chunk, every operation in FP64, the terms as given.
 // Row: [value, N0, Nbkg, d/d(term k, primitive m, slot q)...].
 // ---------------------------------------------------------------------------------------------
 // MODE 2 and 3: the Gauss-Newton product H v of chi^2 and -2lnL for the direction v of the

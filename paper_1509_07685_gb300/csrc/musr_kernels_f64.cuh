@@ -107,10 +107,11 @@ __device__ __forceinline__ double count_weight(double d, bool f32) {
 // that ln x = k ln 2 - ln c + ln(1 + r), r = m c - 1, |r| < h = 2^-11, the last by its series to r^4 with
 // r^5 / 5 folded into the cubic term as (3/20) h^2 r^3: what is left is below 2^-59 on [-h, h] and odd, so
 // that it does not add up over a sum of bins.  One interval holds 1 (h/2 below it, h above) with c = 1, so
-// that ln is exactly 0 there and the absolute error near it stays at 2^-53 |ln x| + 2^-57.  Measured on the host over 65536 Poisson bins of 1e5 / 1e6 / 1e7 counts: a -2lnL's relative error
-// 2.3e-14 / 4.7e-13 / 2.9e-12, those of log(d / N) itself; with c = 1 from 1 to 2^-10 above it, where r leaves
-// [-h, h], and the plain series 4.5e-13 / 1.1e-11 / 4.3e-11.  Arguments
-// outside [2^-1000, 2^1000] (or not positive numbers) take CUDA's log.
+// that ln is exactly 0 there and the absolute error near it stays at 2^-53 |ln x| + 2^-57 (elsewhere three
+// roundings: 2.2 x 2^-53 |ln x| at most).  Over 65536 Poisson bins of 1e5 / 1e6 / 1e7 counts a -2lnL's relative
+// error is 2.3e-14 / 4.7e-13 / 2.9e-12 (a model of these operations on the host), that of log(d / N) itself; with
+// an interval from 1 to 2^-10 above it and c = 1, where r leaves [-h, h], and the plain series it was 4.5e-13 /
+// 1.1e-11 / 4.3e-11.  Arguments outside [2^-1000, 2^1000] (or not positive numbers) take CUDA's log.
 constexpr int kLogOff = 0x3fe6a200;  // high word of the table's lower end
 __device__ __forceinline__ double ln_tab(double x, const double2* tab) {
   const int hi = __double2hiint(x);
