@@ -532,7 +532,8 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
 #pragma unroll
     for (int m = 0; m < M; ++m) V[m] = 0.0;
 
-    if (n >= nlo && n < nhi && dbg_ok(job.dbg, n < hs.stride, kDbgRow)) {
+    const bool in = n >= nlo && n < nhi && dbg_ok(job.dbg, n < hs.stride, kDbgRow);
+    if (in) {
 #pragma unroll
       for (int hl = 0; hl < G; ++hl) {
         if (hl >= nh) break;
@@ -596,7 +597,7 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
         }
       }
     }
-    if (GRAD) {
+    if (GRAD && in) {  // beyond the window a growing factor may have overflowed, and 0 times it is not 0
       const double h2 = 0.5 * t * t;
 #pragma unroll
       for (int k = 0; k < NT; ++k) {

@@ -32,7 +32,7 @@ def _check(p, mode=1):
         ref = oracle.cost(p, p.truth, mode)
         assert np.isfinite(ref[0])
         v, g, st = ctx.eval(p.truth, mode, B.MUSR_FP64)
-        assert st == B.MUSR_OK
+        assert st == B.MUSR_OK and np.all(np.isfinite(g))
         _check_fp64(v, g, ref)
         assert ctx.eval(p.truth, mode, B.MUSR_FP64, grad=False)[0] == v
 
@@ -83,5 +83,19 @@ def test_rates_whose_combination_overflows(musr_lib, shape, lam, sigma):
     terms = [[("AMP", (2,)), ("EXP", (3,)), ("EXP", (3,))]] if shape == "rates" else TERMS[shape]
     counts = np.random.default_rng(8).poisson(3.0, size=(2, 300)).astype(np.float64)
     p = _problem(terms, counts, [4.0, 1.5, 0.3, lam, 3.0, 17.0, sigma])
+    for mode in (0, 1):
+        _check(p, mode)
+
+
+@pytest.mark.parametrize("prim", ["EXP", "LKT"])
+def test_factors_that_overflow_past_the_window(musr_lib, prim):
+    """A growing factor that stays finite up to the last bin (its amplitude keeps N near 1) and overflows within
+    the rest of a CTA iteration: the bins past the window leave the gradient alone."""
+    nbins, dt = 300, 0.5
+    rate = -700.0 / (nbins * dt)
+    a = 1e-290 if prim == "EXP" else 1e-293
+    counts = np.random.default_rng(9).poisson(20.0, size=(2, nbins)).astype(np.float64)
+    terms = [[("AMP", (2,)), (prim, (3,))], [("AMP", (6,)), ("EXP", (4,))]]
+    p = _problem(terms, counts, [2.0, 1.5, a, rate, 0.3, 17.0, 0.2], dt=dt)
     for mode in (0, 1):
         _check(p, mode)
