@@ -202,8 +202,7 @@ __global__ void __launch_bounds__(kBlock, 1) gram64_kernel(const __grid_constant
           } else {
             if (!positive(d)) continue;
             if (!positive(N)) bad = 1;
-            const double y = recip_any(N);
-            w = 2.0 * d * y * y;
+            w = 2.0 * likelihood_weight(d, N);
           }
 #pragma unroll
           for (int i = 0; i < NJ; ++i) {

@@ -102,6 +102,12 @@ __device__ __forceinline__ double count_weight(double d, bool f32) {
   return above_one(d) ? recip(d) : 1.0;
 }
 
+// d / N^2: 0 where N^2 overflows (N from 2^512), as the quotient itself.
+__device__ __forceinline__ double likelihood_weight(double d, double N) {
+  const double y = recip_any(N);
+  return static_cast<unsigned>(__double2hiint(N) - 0x5ff00000) < 0x20000000u ? 0.0 : d * y * y;
+}
+
 // ln x by table and series (Tang's method, ACM TOMS 16 (1990) 378): x = 2^k m with m in
 // [0.70, 1.41); c of m's interval (1/1024 of an octave's mantissa range) approximates 1/m, so
 // that ln x = k ln 2 - ln c + ln(1 + r), r = m c - 1, |r| < h = 2^-11, the last by its series to r^4 with
@@ -559,8 +565,7 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
             cw = 0.0;
             if (positive(d)) {
               if (!positive(N)) bad = 1;
-              const double y = recip_any(N);
-              cw = d * y * y;
+              cw = likelihood_weight(d, N);
             }
           }
           u = cw * Nd;

@@ -94,3 +94,14 @@ def test_matrix_scratch_is_given_back_within_a_budget(musr_lib):
         ref = oracle.cost(p, X[i], 1)
         assert abs(got[0][i] - ref[0]) <= 1e-12 * abs(ref[0])
         assert np.all(np.abs(got[1][i] - ref[1]) <= 1e-12 * ref[2] + 1e-300)
+
+
+@pytest.mark.parametrize("top", [150.0, 160.0, 200.0, 290.0])
+def test_weights_of_a_model_that_grows_beyond_its_square(musr_lib, top):
+    """N from 1 to 10^top within the window: 2 d / N^2 is 0 where N^2 overflows."""
+    nbins, dt = 900, 0.02
+    rate = -np.log(10.0) * top / (nbins * dt)
+    p = mi.Problem(_counts(2, nbins), np.zeros(2), dt * 1000.0, (0.0, nbins * dt),
+                   [[("AMP", (2,)), ("EXP", (3,))]], np.array([[0, 1, 2, 3]] * 2, np.int32), np.zeros(1), 4,
+                   np.array([30.0, 1.5, 0.4, rate]), ["N0", "Nbkg", "A", "lambda"])
+    _check(p, modes=(1,))
