@@ -200,9 +200,11 @@ __global__ void __launch_bounds__(kBlock, 1) gram64_kernel(const __grid_constant
           if (gp.mode == 2) {
             w = 2.0 * (cc.roww[hl] ? __ldg(static_cast<const double*>(cc.roww[hl]) + n) : count_weight(d, f32));
           } else {
-            if (!positive(d)) continue;
-            if (!positive(N)) bad = 1;
-            w = 2.0 * likelihood_weight(d, N);
+            w = 0.0;  // without a count: 0 times a derivative that is not finite is not 0
+            if (positive(d)) {
+              if (!positive(N)) bad = 1;
+              w = 2.0 * likelihood_weight(d, N);
+            }
           }
 #pragma unroll
           for (int i = 0; i < NJ; ++i) {

@@ -105,3 +105,20 @@ def test_weights_of_a_model_that_grows_beyond_its_square(musr_lib, top):
                    [[("AMP", (2,)), ("EXP", (3,))]], np.array([[0, 1, 2, 3]] * 2, np.int32), np.zeros(1), 4,
                    np.array([30.0, 1.5, 0.4, rate]), ["N0", "Nbkg", "A", "lambda"])
     _check(p, modes=(1,))
+
+
+def test_matrix_of_an_undefined_cost_is_refused(musr_lib):
+    """A model that overflows in bins without a count: the cost is infinite, and the matrix refused as the products
+    are."""
+    from paper_1509_07685_gb300 import binding as B
+    counts = _counts(2, 600)
+    counts[:, 300:] = 0.0
+    p = mi.Problem(counts, np.zeros(2), 20.0, (0.0, 12.0), [[("AMP", (2,)), ("EXP", (3,))]],
+                   np.array([[0, 1, 2, 3]] * 2, np.int32), np.zeros(1), 4, np.array([30.0, 1.5, 0.4, -90.0]),
+                   ["N0", "Nbkg", "A", "lambda"])
+    with B.Context(p) as ctx:
+        assert ctx.eval(p.truth, 1, B.MUSR_FP64)[2] == B.MUSR_ENONFINITE
+        assert ctx.gn_product(p.truth, np.eye(4), 1, B.MUSR_FP64)[2] == B.MUSR_ENONFINITE
+        with pytest.raises(B.MusrError) as e:
+            ctx.gauss_newton(p.truth, 1, B.MUSR_FP64)
+        assert e.value.status == B.MUSR_ENONFINITE
