@@ -326,18 +326,20 @@ __device__ void load_chunk64(const Job& job, const HistSet& hs, SM& sm) {
       c.gdot[tid][i] = gd[i];
     }
   } else if (tid == 32) {
-    // The products hold where nothing grows along the steps from an underflowed value and no
-    // factor overflows: every exponent within +-600 over the fit's times, or terms that decay after
-    // time zero and grow by at most that before it.  (Otherwise, and for NaN parameters, every bin is evaluated afresh.)
+    // The products hold where no factor of them overflows and nothing grows from an underflowed value: every
+    // exponent within +-600 over the fit's times and the steps from a fresh bin (up to len further), or terms
+    // that decay after time zero and whose fresh value and cross term exp(-S t i D) before it stay within
+    // that.  (Otherwise, and for NaN parameters, every bin is evaluated afresh.)
     const double t1 = (cc.nlo - 4 - cc.t0) * hs.dt_us, t2 = (cc.nhi - cc.t0) * hs.dt_us;
-    const double T = fmax(fabs(t1), fabs(t2)) + D, T0 = fmax(-t1, 0.0);  // T0: the stretch before time zero
+    const double len = fmin(kRebase * D, t2 - t1 + D);
+    const double T = fmax(fabs(t1), fabs(t2)) + D + len, T0 = fmax(-t1, 0.0);  // T0: the stretch before time zero
     int ok = T0 * c.rate <= 600.0;
     for (int k = 0; k < hs.nterms && k < kMaxTerms; ++k) {
       const double kt = c.kt[k], S = c.S[k] + (c.kinds[k] == kTermKT ? kt * kt : 0.0);
       const double lam = fabs(c.lam[k]) + (c.kinds[k] == kTermLKT ? fabs(kt) : 0.0);
       const bool small = lam * T + S * T * T <= 600.0;
       const bool decays = c.lam[k] >= 0.0 && (c.kinds[k] != kTermLKT || kt >= 0.0) && lam < 1e150 && S < 1e150 &&
-                          lam * T0 + S * T0 * (T0 + D) <= 600.0;
+                          lam * T0 + S * T0 * (T0 + len) <= 600.0;
       if (!(small || decays)) ok = 0;
     }
     c.safe = ok;

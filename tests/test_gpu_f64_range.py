@@ -99,3 +99,24 @@ def test_factors_that_overflow_past_the_window(musr_lib, prim):
     p = _problem(terms, counts, [2.0, 1.5, a, rate, 0.3, 17.0, 0.2], dt=dt)
     for mode in (0, 1):
         _check(p, mode)
+
+
+@pytest.mark.parametrize("lam,sigma,kt,t0", [(0.4, 48.8, 0.5, 3.0), (0.4, 0.3, 48.8, 3.0), (0.4, 90.0, 0.1, 1.0),
+                                             (0.2, 12.0, 12.0, 40.25), (-11.5, 0.1, 0.1, 1600.0),
+                                             (0.1, 1.3, 1.3, 1600.0)])
+def test_factors_taken_over_many_steps(musr_lib, lam, sigma, kt, t0):
+    """Rates whose factors a thread takes over up to 31 steps of 256 bins from a bin before time zero, where the
+    cross term of a Gaussian grows with every step: a batch of vectors, whose tiles hold that many steps."""
+    from paper_1509_07685_gb300 import binding as B
+    terms = [[("AMP", (2,)), ("EXP", (3,)), ("GAUSS", (6,))], [("AMP", (2,)), ("KT", (4,))]]
+    counts = np.random.default_rng(10).poisson(9.0, size=(3, 3150)).astype(np.float64)
+    p = _problem(terms, counts, [4.0, 1.5, 0.1, lam, kt, 17.0, sigma], dt=0.0103, fit=(-40.0, 40.0))
+    p.t0[:] = t0
+    X = np.stack([p.truth] * 700)
+    with B.Context(p) as ctx:
+        for mode in (0, 1):
+            ref = oracle.cost(p, p.truth, mode)
+            vals, grads, st = ctx.eval_batch(X, mode, B.MUSR_FP64)
+            assert st == B.MUSR_OK and np.isfinite(ref[0]) and np.all(np.isfinite(grads))
+            for i in (0, 699):
+                _check_fp64(vals[i], grads[i], ref)
