@@ -23,7 +23,7 @@
 //
 // Measured on GB300 (256 x 256 x 128, device arrays): 15.33 -> 6.16 ms a solve (z 0.43 + 0.44, y 0.88 +
 // 0.91, x 3.50 ms; 26 FP64 instructions per point of a y transform, 55 per point of the x convolution;
-// the pipe 83-86 % of its peak busy; DRAM below 0.3 TB/s).  37 x 44 x 23: 189 -> 64 us.
+// the pipe 83-86 % of its peak busy; DRAM below 0.5 TB/s).  37 x 44 x 23: 189 -> 64 us.
 //
 // The half length mp is the product of 2, 3, 5 and 7 at or above m that needs the fewest
 // instructions (m itself where it is such a product): the padded circular length 2 mp >= 2 m gives

@@ -5,14 +5,15 @@
 // The matrix by products with unit vectors is P evaluations: 31 FP64 instructions per (histogram,
 // bin) pair and parameter, 862 for 28 parameters, and the FP64 pipe was 91 % busy with them.  A
 // histogram has few local slots (7 there), so its own triangle of 28 sums, with the 13 multiply-adds
-// that form J, the reciprocal and the weight, is 57 per pair.
+// that form J, the reciprocal and the weight, is 57 per pair (90 executed, with the
+// time functions, the set-up and the sums).
 // The CTA's threads first evaluate the time functions of 256 bins (the basis functions, and P t,
 // P t^2 and the Kubo-Toyabe derivatives of each term) into shared memory, a bin each; then each
 // warp takes one histogram of the chunk (several warps one histogram where the chunk has fewer than
 // 8) and a lane a bin, with the triangle in registers; so one kernel per shape serves every theory,
 // J's coefficients being data.  A CTA keeps its sums over all its tiles of a chunk and writes one row.
 // Measured on GB300 (8 x 65536 bins, 28 parameters, -2lnL, the whole call): 8.88 ms with the term-list
-// kernel's products, 0.85 ms with the basis kernel's, 0.137 ms here.
+// kernel's products, 0.85 ms with the basis kernel's, 0.134 ms here.
 // Up to 12 local slots (78 sums fill the registers); theories with more, and dynamic Kubo-Toyabe factors,
 // whose tables are solved for a job on the device, keep the products, as do theories with a primitive on
 // N0's slot.

@@ -674,10 +674,10 @@ __device__ void basis64_item(const Job& job, const HistSet& hs, int item, Smem64
 // Measured on GB300 (a call with its copies, before: the term-list kernel with CUDA's library
 // functions per histogram and bin):
 //   8 x 65536 bins, two cosine terms, -2lnL value and gradient, one vector   467 ->   79 us
-//   1 x 16384 bins, one cosine term, -2lnL at 1000 vectors                  4116 -> 1050 us
+//   1 x 16384 bins, one cosine term, -2lnL at 1000 vectors                  4116 -> 1040 us
 //   8 x 65536 bins, Gauss-Newton products along 28 directions               8884 ->  849 us
 //   (the whole matrix: musr_gram64.cu)
-// The first of these executes 46 FP64 instructions per pair (16 of them fresh time factors, a CTA
+// The first of these executes 44 FP64 instructions per pair (16 of them fresh time factors, a CTA
 // having two iterations), the second 30 (33, 1114 us, with a table of 256 intervals and the bin's time
 // formed in every bin), the third 31.
 template <int SHAPE, int MODE, bool GRAD>
