@@ -857,7 +857,10 @@ struct LaunchPlan {
 int refuse_capture(musr_ctx* ctx) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const cudaError_t e = cudaStreamIsCapturing(ctx->stream, &cap);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaStreamIsCapturing");
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // not left for the next launch to find
+    return cuda_fail(ctx, e, "cudaStreamIsCapturing");
+  }
   if (cap == cudaStreamCaptureStatusNone) return MUSR_OK;
   return fail(ctx, MUSR_ESTATE, "the context's stream is capturing and the call needs set-up (tables, buffers): make "
                                 "the same call once before the capture");
